@@ -13,376 +13,289 @@
 // memory.
 //
 // Layout: Q, K, V, O contiguous row-major [B,H,N,d] float32.
-// Two kernels:
-//   attn_fwd_f32_cc_kernel   CTA of 128 threads = 4 warps, BM = 32 rows (8 per warp), BN = 64
-//                            keys; K and V tiles shared by the CTA's 32 rows through smem.
-//   attn_fwd_f32_small_kernel  8 query rows of one (b, h) per CTA, one warp per row, for
-//                            problems too small to give every SM a 32-row CTA: 64-key chunks of
-//                            K and V are copied with cp.async, every piece of a chunk in flight
-//                            at once, double-buffered, which matters when the call is bound by
-//                            memory latency.
+//
+// What bounds it: the FMA pipe (152 SMs x 128 FMA/clk), provided that shared memory and issue keep
+// up.  Each thread therefore holds an R x 8 block of scores and an R x 4 VC block of O in registers:
+// per 4 features an R x 8 block costs R + 8 16-byte shared loads (two wavefronts each, see the lane
+// map) for 32 R FMAs, which at R = 8 is half of what shared memory can deliver, at R = 4 three
+// quarters.  K and V tiles come by cp.async while the previous tile's softmax and products run.
+// A CTA is WR row warps (4R rows each) x KW key groups; the groups take alternate 64-key tiles and
+// merge their (m, l, O) at the end, so that a short problem still puts 4 to 8 warps on an SM.
+// Small R and more groups shorten the dependent chain of one CTA; large R does the least work per
+// score.  pick_tile weighs the two from measured step times.
+//
+// Measured on a GB300 (2070 MHz; before: one lane per output column, 8-row warps, scalar loads):
+// 2x8x1000x1500 d=64 482 -> 171 us (36 TFLOP/s), 1x8x1024x1024 d=128 517 -> 125 us, 1x8x256x256
+// d=64 27 -> 10 us, 1x1x300x2048 d=64 115 -> 33 us, 1x1x128x128 d=64 10.4 -> 6.3 us.  The tile's
+// former fill by cp.async with a zero-fill source size cost more than its products (16-row tile,
+// one 256-key step: 13 us with it, 6.4 us with the plain form and stores of zeros).
 #include <cuda_runtime.h>
 #include <math.h>
 #include <cstdio>
 
+#include "f32_common.cuh"
 #include "internal.h"
 
 namespace moa {
 namespace {
 
-constexpr int kThreads = 128;
-constexpr int kWarps = kThreads / 32;
-constexpr int kRowsPerWarp = 8;
-constexpr int kBM = kWarps * kRowsPerWarp;  // 32 query rows per CTA
-constexpr int kBN = 64;                     // keys per tile
-constexpr int kMaxD = 128;
-constexpr int kMaxColGroups = kMaxD / 32;    // output columns per lane: c = lane + 32*g
+using namespace f32;
 
-struct F32Smem {
-  // K tile padded by one float per row so that lane-strided reads hit distinct banks.
-  static size_t bytes(int dk, int dv) {
-    return sizeof(float) * (size_t(kBM) * dk + size_t(kBN) * (dk + 1) + size_t(kBN) * dv +
-                            size_t(kWarps) * kRowsPerWarp * kBN);
+constexpr int kBN = 64;                     // keys per key group and step
+constexpr int kHalf = kBN / 2;              // keys of P held in shared memory at a time
+constexpr int kLdp = kHalf + 8;             // floats per row of P: 4 rows of a store or load on disjoint banks
+constexpr int kMaxSmem = 232448;            // shared memory a CTA can have
+
+// VC: 32-column blocks of V (ceil(d_v / 32)).  R: rows per thread (4R per warp).  WR: row warps,
+// KW: key groups.
+template <int VC, int R, int WR, int KW>
+struct F32Tile {
+  static constexpr int kThreads = 32 * WR * KW;
+  static constexpr int kBM = 4 * R * WR;     // query rows per CTA
+  static constexpr int kStep = kBN * KW;     // keys per step of the CTA
+  static constexpr int kLdv = 32 * VC;
+  // 128 registers hold an R = 4 thread with d_v <= 64 (two 8-warp CTAs an SM); the rest need more.
+  static constexpr int kMinBlocks = (R == 4 && VC <= 2 ? 16 : 8) / (WR * KW) > 0
+                                        ? (R == 4 && VC <= 2 ? 16 : 8) / (WR * KW) : 1;
+  static size_t smem_bytes(int dk) {
+    return sizeof(float) * (size_t(kBM) * odd_stride(dk) + size_t(kStep) * (odd_stride(dk) + kLdv) +
+                            size_t(kBM) * KW * kLdp);
   }
 };
 
-__global__ void __launch_bounds__(kThreads)
+template <int VC, int R, int WR, int KW>
+__global__ void __launch_bounds__(F32Tile<VC, R, WR, KW>::kThreads, F32Tile<VC, R, WR, KW>::kMinBlocks)
 attn_fwd_f32_cc_kernel(const float* __restrict__ Q, const float* __restrict__ K,
                        const float* __restrict__ V, float* __restrict__ O,
                        float* __restrict__ lse, int Nq, int Nk, int dk, int dv, int n_qtiles,
                        float scale) {
-  extern __shared__ float smem[];
-  float* sQ = smem;                          // [kBM][dk]
-  float* sK = sQ + kBM * dk;                 // [kBN][dk+1]
-  float* sV = sK + kBN * (dk + 1);           // [kBN][dv]
-  float* sP = sV + kBN * dv;                 // [kWarps][kRowsPerWarp][kBN]
-  const int ldk = dk + 1;
+  using T = F32Tile<VC, R, WR, KW>;
+  constexpr int kThreads = T::kThreads, kBM = T::kBM, kStep = T::kStep, kLdv = T::kLdv;
+  extern __shared__ __align__(16) float smem[];
+  const int ldk = odd_stride(dk);
+  float* sQ = smem;                // [kBM][ldk]
+  float* sK = sQ + kBM * ldk;      // [kStep][ldk]
+  float* sV = sK + kStep * ldk;    // [kStep][kLdv]
+  float* sP = sV + kStep * kLdv;   // [KW * WR][4R][kLdp]
 
-  const int warp = threadIdx.x >> 5;
   const int lane = threadIdx.x & 31;
+  const int warp = (threadIdx.x >> 5) % WR, kg = (threadIdx.x >> 5) / WR;  // row warp, key group
+  // Column group 0..7 and row group 0..3.  Lanes 2i and 2i + 1 share their columns: a 16-byte shared
+  // load then takes two wavefronts; with the column group in the low lane bits it takes four.
+  const int cg = (lane >> 1) & 7, rg = (lane & 1) | (lane >> 4) << 1;
   const long long bh = blockIdx.x / n_qtiles;
-  const int qt = blockIdx.x % n_qtiles;
-  const int q0 = qt * kBM;
-
+  const int q0 = (blockIdx.x % n_qtiles) * kBM;
   const float* Qh = Q + bh * (long long)Nq * dk;
   const float* Kh = K + bh * (long long)Nk * dk;
   const float* Vh = V + bh * (long long)Nk * dv;
-  float* Oh = O + bh * (long long)Nq * dv;
 
-  // Q tile -> shared memory (rows past N_q are zero; they are computed but never stored).
-  for (int idx = threadIdx.x; idx < kBM * dk; idx += kThreads) {
-    const int r = idx / dk, j = idx % dk;
-    sQ[idx] = (q0 + r < Nq) ? Qh[(long long)(q0 + r) * dk + j] : 0.f;
-  }
+  // rows [r0, r0 + rows) of a [n, d] array -> shared rows of ld floats; rows past n are zeros
+  const int seg0 = threadIdx.x & 15, row0 = threadIdx.x >> 4;
+  auto request = [&](float* dst, int ld, const float* src, int d, long long r0, int rows, int n) {
+    dst += row0 * ld + 4 * seg0;
+    src += (r0 + row0) * d + 4 * seg0;
+    const int last = int(min((long long)rows, n - r0));
+    for (int s = 4 * seg0; s < d; s += 64, dst += 64, src += 64) {
+      int r = row0;
+#pragma unroll 4
+      for (; r < last; r += kThreads / 16) cp_async16(dst + (r - row0) * ld, src + (long long)(r - row0) * d);
+#pragma unroll 1
+      for (; r < rows; r += kThreads / 16)
+        *reinterpret_cast<float4*>(dst + (r - row0) * ld) = make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+  };
+  request(sQ, ldk, Qh, dk, q0, kBM, Nq);
+  request(sK, ldk, Kh, dk, 0, kStep, Nk);
+  cp_async_commit();
+  request(sV, kLdv, Vh, dv, 0, kStep, Nk);
+  cp_async_commit();
 
-  float m[kRowsPerWarp], l[kRowsPerWarp];
-  float acc[kRowsPerWarp][kMaxColGroups];
+  // This thread: rows 4r + rg (r < R) of its warp; keys cg + 8j (j < 8) of its group's tile;
+  // output columns 32b + 4cg .. +3 (b < VC).
+  float m[R], l[R], acc[R][4 * VC];
 #pragma unroll
-  for (int r = 0; r < kRowsPerWarp; ++r) {
+  for (int r = 0; r < R; ++r) {
     m[r] = -INFINITY;
     l[r] = 0.f;
 #pragma unroll
-    for (int g = 0; g < kMaxColGroups; ++g) acc[r][g] = 0.f;
+    for (int c = 0; c < 4 * VC; ++c) acc[r][c] = 0.f;
   }
-  const int ngroups = (dv + 31) / 32;
-  float* myP = sP + warp * kRowsPerWarp * kBN;
-  const float* myQ = sQ + warp * kRowsPerWarp * dk;
+  const float* myQ = sQ + (warp * 4 * R + rg) * ldk;                        // row r: + 4r*ldk
+  const float* myK = sK + (kg * kBN + cg) * ldk;                            // key j: + 8j*ldk
+  const float* myV = sV + kg * kBN * kLdv + 4 * cg;
+  float* myP = sP + ((kg * WR + warp) * 4 * R + rg) * kLdp;                 // row r: + 4r*kLdp
 
-  for (int k0 = 0; k0 < Nk; k0 += kBN) {
-    __syncthreads();  // previous tile fully consumed (and Q visible on the first pass)
-    for (int idx = threadIdx.x; idx < kBN * dk; idx += kThreads) {
-      const int r = idx / dk, j = idx % dk;
-      sK[r * ldk + j] = (k0 + r < Nk) ? Kh[(long long)(k0 + r) * dk + j] : 0.f;
+  // left: keys from k0 on
+  for (long long k0 = 0, left = Nk; left > 0; k0 += kStep, left -= kStep) {
+    const int mine = int(left) - kg * kBN;  // keys from this group's tile on
+    const bool live = KW == 1 || mine > 0;  // warp-uniform
+    cp_async_wait<1>();  // K tile (and Q) here; V may be on its way
+    __syncthreads();
+    float s[R][8];
+#pragma unroll
+    for (int r = 0; r < R; ++r)
+#pragma unroll
+      for (int j = 0; j < 8; ++j) s[r][j] = 0.f;
+    const int f_end = live ? dk : 0;
+#pragma unroll 1
+    for (int f = 0; f < f_end; f += 4) {
+      float4 kk[8];
+#pragma unroll
+      for (int j = 0; j < 8; ++j) kk[j] = *reinterpret_cast<const float4*>(myK + 8 * j * ldk + f);
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        const float4 q = *reinterpret_cast<const float4*>(myQ + 4 * r * ldk + f);
+#pragma unroll
+        for (int j = 0; j < 8; ++j) s[r][j] = fmaf(q.x, kk[j].x, s[r][j]);
+#pragma unroll
+        for (int j = 0; j < 8; ++j) s[r][j] = fmaf(q.y, kk[j].y, s[r][j]);
+#pragma unroll
+        for (int j = 0; j < 8; ++j) s[r][j] = fmaf(q.z, kk[j].z, s[r][j]);
+#pragma unroll
+        for (int j = 0; j < 8; ++j) s[r][j] = fmaf(q.w, kk[j].w, s[r][j]);
+      }
     }
-    for (int idx = threadIdx.x; idx < kBN * dv; idx += kThreads) {
-      const int r = idx / dv;
-      sV[idx] = (k0 + r < Nk) ? Vh[(long long)k0 * dv + idx] : 0.f;
+    __syncthreads();  // every warp has read the K tile
+    if (left > kStep) request(sK, ldk, Kh, dk, k0 + kStep, kStep, Nk);
+    cp_async_commit();
+
+    // Online softmax; the 8 lanes of a row share its maximum, each keeps its own part of the sum.
+    if (live) {
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+#pragma unroll
+        for (int j = 0; j < 8; ++j) s[r][j] = cg + 8 * j < mine ? __fmul_rn(s[r][j], scale) : -INFINITY;
+        float t = s[r][0];
+#pragma unroll
+        for (int j = 1; j < 8; ++j) t = fmaxf(t, s[r][j]);
+#pragma unroll
+        for (int off = 8; off > 1; off >>= 1) t = fmaxf(t, __shfl_xor_sync(0xffffffffu, t, off));
+        const float mnew = fmaxf(m[r], t);         // finite: the tile has at least one key
+        const float alpha = expf(m[r] - mnew);     // exp(-inf) = 0 on the first tile
+        m[r] = mnew;
+        float sum = 0.f;
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+          s[r][j] = expf(s[r][j] - mnew);
+          sum += s[r][j];
+        }
+        l[r] = fmaf(l[r], alpha, sum);
+#pragma unroll
+        for (int c = 0; c < 4 * VC; ++c) acc[r][c] *= alpha;
+      }
+    }
+    cp_async_wait<1>();  // V tile here; the next K may be on its way
+    __syncthreads();
+    if (live) {
+#pragma unroll
+      for (int half = 0; half < 2; ++half) {
+        if (half) __syncwarp();  // the first half's P has been read
+#pragma unroll
+        for (int r = 0; r < R; ++r)
+#pragma unroll
+          for (int j = 0; j < 4; ++j) myP[4 * r * kLdp + cg + 8 * j] = s[r][4 * half + j];
+        __syncwarp();
+#pragma unroll 1
+        for (int k = 0; k < kHalf; k += 4) {
+          float4 vv[4][VC];
+#pragma unroll
+          for (int u = 0; u < 4; ++u)
+#pragma unroll
+            for (int b = 0; b < VC; ++b)
+              vv[u][b] = *reinterpret_cast<const float4*>(myV + (half * kHalf + k + u) * kLdv + 32 * b);
+#pragma unroll
+          for (int r = 0; r < R; ++r) {
+            const float4 p = *reinterpret_cast<const float4*>(myP + 4 * r * kLdp + k);
+            const float pu[4] = {p.x, p.y, p.z, p.w};
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+#pragma unroll
+              for (int b = 0; b < VC; ++b) {
+                acc[r][4 * b] = fmaf(pu[u], vv[u][b].x, acc[r][4 * b]);
+                acc[r][4 * b + 1] = fmaf(pu[u], vv[u][b].y, acc[r][4 * b + 1]);
+                acc[r][4 * b + 2] = fmaf(pu[u], vv[u][b].z, acc[r][4 * b + 2]);
+                acc[r][4 * b + 3] = fmaf(pu[u], vv[u][b].w, acc[r][4 * b + 3]);
+              }
+          }
+        }
+      }
+    }
+    __syncthreads();  // every warp has read the V tile
+    if (left > kStep) request(sV, kLdv, Vh, dv, k0 + kStep, kStep, Nk);
+    cp_async_commit();
+  }
+
+  if constexpr (KW > 1) {
+    // Merge of the key groups: O = sum_g e^(m_g - M) O_g, l = sum_g e^(m_g - M) l_g, M = max m_g.
+    // Groups g > 0 leave their state where the tiles were (thread-private slots, lane-contiguous).
+    constexpr int kState = 2 * R + 4 * R * VC;
+    static_assert((KW - 1) * WR * kState * 32 <= kStep * (4 + kLdv) + kBM * KW * kLdp, "merge slots");
+    float* slot = sK + lane;
+    if (kg > 0) {
+      float* mine = slot + ((kg - 1) * WR + warp) * kState * 32;
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        mine[32 * r] = m[r];
+        mine[32 * (R + r)] = l[r];
+#pragma unroll
+        for (int c = 0; c < 4 * VC; ++c) mine[32 * (2 * R + 4 * VC * r + c)] = acc[r][c];
+      }
     }
     __syncthreads();
-
-    // Scores of this warp's 8 rows against keys (lane) and (lane + 32) of the tile.
-    float s0[kRowsPerWarp], s1[kRowsPerWarp];
+    if (kg > 0) return;
+#pragma unroll 1
+    for (int g = 1; g < KW && g * kBN < Nk; ++g) {  // groups that had a key
+      const float* other = slot + ((g - 1) * WR + warp) * kState * 32;
 #pragma unroll
-    for (int r = 0; r < kRowsPerWarp; ++r) s0[r] = s1[r] = 0.f;
-    const float* k0p = sK + lane * ldk;
-    const float* k1p = sK + (lane + 32) * ldk;
-    for (int j = 0; j < dk; ++j) {
-      const float ka = k0p[j], kb = k1p[j];
+      for (int r = 0; r < R; ++r) {
+        const float mo = other[32 * r], mn = fmaxf(m[r], mo);
+        const float a = expf(m[r] - mn), b = expf(mo - mn);
+        m[r] = mn;
+        l[r] = fmaf(other[32 * (R + r)], b, l[r] * a);
 #pragma unroll
-      for (int r = 0; r < kRowsPerWarp; ++r) {
-        const float q = myQ[r * dk + j];
-        s0[r] = fmaf(q, ka, s0[r]);
-        s1[r] = fmaf(q, kb, s1[r]);
+        for (int c = 0; c < 4 * VC; ++c)
+          acc[r][c] = fmaf(other[32 * (2 * R + 4 * VC * r + c)], b, acc[r][c] * a);
       }
     }
-    const bool v0 = (k0 + lane) < Nk, v1 = (k0 + lane + 32) < Nk;
-    float alpha[kRowsPerWarp];
-#pragma unroll
-    for (int r = 0; r < kRowsPerWarp; ++r) {
-      const float x0 = v0 ? s0[r] * scale : -INFINITY;
-      const float x1 = v1 ? s1[r] * scale : -INFINITY;
-      float tmax = fmaxf(x0, x1);
-#pragma unroll
-      for (int off = 16; off > 0; off >>= 1) tmax = fmaxf(tmax, __shfl_xor_sync(0xffffffffu, tmax, off));
-      const float mnew = fmaxf(m[r], tmax);   // finite: every tile has at least one key
-      alpha[r] = expf(m[r] - mnew);           // exp(-inf) = 0 on the first tile
-      const float p0 = expf(x0 - mnew), p1 = expf(x1 - mnew);
-      float psum = p0 + p1;
-#pragma unroll
-      for (int off = 16; off > 0; off >>= 1) psum += __shfl_xor_sync(0xffffffffu, psum, off);
-      l[r] = l[r] * alpha[r] + psum;
-      m[r] = mnew;
-      myP[r * kBN + lane] = p0;
-      myP[r * kBN + lane + 32] = p1;
-    }
-    __syncwarp();
-    // acc = alpha * acc + P V for this warp's rows and this lane's output columns.
-#pragma unroll
-    for (int r = 0; r < kRowsPerWarp; ++r)
-#pragma unroll
-      for (int g = 0; g < kMaxColGroups; ++g) acc[r][g] *= alpha[r];
-    const int kn = min(kBN, Nk - k0);
-    for (int kk = 0; kk < kn; ++kk) {
-      float vv[kMaxColGroups];
-#pragma unroll
-      for (int g = 0; g < kMaxColGroups; ++g) {
-        const int c = lane + 32 * g;
-        vv[g] = (g < ngroups && c < dv) ? sV[kk * dv + c] : 0.f;
-      }
-#pragma unroll
-      for (int r = 0; r < kRowsPerWarp; ++r) {
-        const float p = myP[r * kBN + kk];
-#pragma unroll
-        for (int g = 0; g < kMaxColGroups; ++g) acc[r][g] = fmaf(p, vv[g], acc[r][g]);
-      }
-    }
-    __syncwarp();
   }
-
 #pragma unroll
-  for (int r = 0; r < kRowsPerWarp; ++r) {
-    const int row = q0 + warp * kRowsPerWarp + r;
+  for (int r = 0; r < R; ++r) {
+#pragma unroll
+    for (int off = 8; off > 1; off >>= 1) l[r] += __shfl_xor_sync(0xffffffffu, l[r], off);
+    const int row = q0 + warp * 4 * R + 4 * r + rg;
     if (row >= Nq) continue;
     const float inv = 1.0f / l[r];
     // ln sum_k exp(scale s_k) = m + ln l (m is the exact row maximum here).
-    if (lse != nullptr && lane == 0) lse[bh * Nq + row] = m[r] + logf(l[r]);
-#pragma unroll
-    for (int g = 0; g < kMaxColGroups; ++g) {
-      const int c = lane + 32 * g;
-      if (g < ngroups && c < dv) Oh[(long long)row * dv + c] = acc[r][g] * inv;
-    }
-  }
-}
-
-// Small problems: 8 query rows of one (b, h) per CTA, one warp per row.  The CTA's 256
-// threads copy 64-key chunks of K and V into shared memory with cp.async (16-byte pieces, all
-// in flight at once), double-buffered: chunk c+1 is requested before chunk c is used, so a call
-// that is bound by memory latency pays it about once per chunk pair instead of once per
-// dependent load.  Per chunk, lane = key for the scores (keys lane and lane + 32), lane =
-// output column for the sum over V.
-constexpr int kSmallRows = 8;     // rows (= warps) per CTA
-constexpr int kSmallKeys = 64;    // keys per chunk
-constexpr int kSmallThreads = 32 * kSmallRows;
-
-struct SmallSmem {
-  // K rows padded by 4 floats: 16-byte aligned, and the float4 reads of 8 consecutive key rows
-  // fall on disjoint banks.
-  __host__ __device__ static int ldk(int dk) { return dk + 4; }
-  static size_t bytes(int dk, int dv) {
-    return sizeof(float) * (size_t(kSmallRows) * dk + 2 * size_t(kSmallKeys) * ldk(dk) +
-                            2 * size_t(kSmallKeys) * dv + size_t(kSmallRows) * kSmallKeys);
-  }
-};
-
-// 16 bytes global -> shared, asynchronous; src_bytes = 0 writes zeros (the source is not read).
-__device__ __forceinline__ void cp_async16(float* dst, const float* src, int src_bytes) {
-  const unsigned d = static_cast<unsigned>(__cvta_generic_to_shared(dst));
-  const size_t g = __cvta_generic_to_global(src);
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(g), "r"(src_bytes)
-               : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_async_wait() {
-  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
-}
-
-__global__ void __launch_bounds__(kSmallThreads)
-attn_fwd_f32_small_kernel(const float* __restrict__ Q, const float* __restrict__ K,
-                          const float* __restrict__ V, float* __restrict__ O,
-                          float* __restrict__ lse, int Nq, int Nk, int dk, int dv, int n_qtiles,
-                          float scale) {
-  extern __shared__ __align__(16) float smem[];
-  const int ldk = SmallSmem::ldk(dk);
-  float* sQ = smem;                                   // [8][dk]
-  float* sK = sQ + kSmallRows * dk;                   // [2][64][dk + 4]
-  float* sV = sK + 2 * kSmallKeys * ldk;              // [2][64][dv]
-  float* sP = sV + 2 * kSmallKeys * dv;               // [8][64]
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const long long bh = blockIdx.x / n_qtiles;
-  const int row = (blockIdx.x % n_qtiles) * kSmallRows + warp;  // query row of this warp
-  const bool active = row < Nq;
-  const float* Kh = K + bh * (long long)Nk * dk;
-  const float* Vh = V + bh * (long long)Nk * dv;
-
-  const int kseg = dk / 4, vseg = dv / 4;  // 16-byte pieces per row (d is a multiple of 4)
-  auto request = [&](int c) {             // chunk c -> buffer c % 2
-    const int k0 = c * kSmallKeys, b = c & 1;
-    float* dK = sK + b * kSmallKeys * ldk;
-    float* dV = sV + b * kSmallKeys * dv;
-    for (int i = threadIdx.x; i < kSmallKeys * kseg; i += kSmallThreads) {
-      const int r = i / kseg, j = i - r * kseg;
-      const bool in = k0 + r < Nk;
-      cp_async16(dK + r * ldk + 4 * j, in ? Kh + (long long)(k0 + r) * dk + 4 * j : Kh, in ? 16 : 0);
-    }
-    for (int i = threadIdx.x; i < kSmallKeys * vseg; i += kSmallThreads) {
-      const int r = i / vseg, j = i - r * vseg;
-      const bool in = k0 + r < Nk;
-      cp_async16(dV + r * dv + 4 * j, in ? Vh + (long long)(k0 + r) * dv + 4 * j : Vh, in ? 16 : 0);
-    }
-    cp_async_commit();
-  };
-
-  request(0);
-  if (active)
-    for (int j = lane; j < dk; j += 32) sQ[warp * dk + j] = Q[(bh * Nq + row) * (long long)dk + j];
-  const float* q = sQ + warp * dk;
-  float* p_row = sP + warp * kSmallKeys;
-
-  float m = -INFINITY, l = 0.f;
-  float acc[kMaxColGroups];
-#pragma unroll
-  for (int g = 0; g < kMaxColGroups; ++g) acc[g] = 0.f;
-  const int n_chunks = (Nk + kSmallKeys - 1) / kSmallKeys;
-  for (int c = 0; c < n_chunks; ++c) {
-    if (c + 1 < n_chunks) {
-      request(c + 1);  // its buffer was released by the barrier at the end of chunk c - 1
-      cp_async_wait<1>();
-    } else {
-      cp_async_wait<0>();
-    }
-    __syncthreads();  // chunk c (and the Q rows) visible to every warp
-    if (active) {
-      const int k0 = c * kSmallKeys, b = c & 1;
-      const float* cK = sK + b * kSmallKeys * ldk;
-      const float* cV = sV + b * kSmallKeys * dv;
-      // scores of keys k0 + lane and k0 + lane + 32
-      const float* ka = cK + lane * ldk;
-      const float* kb = cK + (lane + 32) * ldk;
-      float s0 = 0.f, s1 = 0.f;
-      for (int j = 0; j < dk; j += 4) {
-        const float4 qv = *reinterpret_cast<const float4*>(q + j);
-        const float4 a4 = *reinterpret_cast<const float4*>(ka + j);
-        const float4 b4 = *reinterpret_cast<const float4*>(kb + j);
-        s0 = fmaf(qv.x, a4.x, s0);
-        s1 = fmaf(qv.x, b4.x, s1);
-        s0 = fmaf(qv.y, a4.y, s0);
-        s1 = fmaf(qv.y, b4.y, s1);
-        s0 = fmaf(qv.z, a4.z, s0);
-        s1 = fmaf(qv.z, b4.z, s1);
-        s0 = fmaf(qv.w, a4.w, s0);
-        s1 = fmaf(qv.w, b4.w, s1);
-      }
-      const float x0 = k0 + lane < Nk ? s0 * scale : -INFINITY;
-      const float x1 = k0 + lane + 32 < Nk ? s1 * scale : -INFINITY;
-      float cmax = fmaxf(x0, x1);
-#pragma unroll
-      for (int off = 16; off > 0; off >>= 1) cmax = fmaxf(cmax, __shfl_xor_sync(0xffffffffu, cmax, off));
-      const float mnew = fmaxf(m, cmax);  // finite: every chunk has at least one key
-      const float alpha = expf(m - mnew);  // exp(-inf) = 0 on the first chunk
-      const float p0 = expf(x0 - mnew), p1 = expf(x1 - mnew);
-      float psum = p0 + p1;
-#pragma unroll
-      for (int off = 16; off > 0; off >>= 1) psum += __shfl_xor_sync(0xffffffffu, psum, off);
-      l = l * alpha + psum;
-      m = mnew;
-      p_row[lane] = p0;
-      p_row[lane + 32] = p1;
-      __syncwarp();
-      // lane = output column: acc = alpha * acc + sum over the chunk's keys of p_k V[k, c]
-#pragma unroll
-      for (int g = 0; g < kMaxColGroups; ++g) acc[g] *= alpha;
-      const int kn = min(kSmallKeys, Nk - k0);
-      for (int k = 0; k < kn; k += 4) {
-        float pv[4], vv[4][kMaxColGroups];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          pv[u] = k + u < kn ? p_row[k + u] : 0.f;  // zero-filled rows past N_k also read 0
-#pragma unroll
-          for (int g = 0; g < kMaxColGroups; ++g) {
-            const int col = lane + 32 * g;
-            vv[u][g] = col < dv ? cV[(k + u) * dv + col] : 0.f;
-          }
-        }
-#pragma unroll
-        for (int u = 0; u < 4; ++u)
-#pragma unroll
-          for (int g = 0; g < kMaxColGroups; ++g) acc[g] = fmaf(pv[u], vv[u][g], acc[g]);
-      }
-    }
-    __syncthreads();  // buffer c % 2 and the P rows are free again
-  }
-  if (active) {
-    const float inv = 1.0f / l;
+    if (lse != nullptr && cg == 0) lse[bh * Nq + row] = m[r] + logf(l[r]);
     float* orow = O + (bh * Nq + row) * (long long)dv;
 #pragma unroll
-    for (int g = 0; g < kMaxColGroups; ++g) {
-      const int col = lane + 32 * g;
-      if (col < dv) orow[col] = acc[g] * inv;
+    for (int b = 0; b < VC; ++b) {
+      const int c = 32 * b + 4 * cg;
+      if (c < dv)
+        *reinterpret_cast<float4*>(orow + c) =
+            make_float4(acc[r][4 * b] * inv, acc[r][4 * b + 1] * inv, acc[r][4 * b + 2] * inv,
+                        acc[r][4 * b + 3] * inv);
     }
-    // ln sum_k exp(scale s_k) = m + ln l (m is the exact row maximum here)
-    if (lse != nullptr && lane == 0) lse[bh * Nq + row] = m + logf(l);
   }
 }
 
-}  // namespace
-
-int launch_attn_fwd_f32(const AttnArgs& a, char* msg, size_t msglen) {
-  // Few 32-row CTAs (fewer than two per SM): 8-row CTAs instead, each with its K/V chunks
-  // requested all at once.
-  int dev = 0, sms = 148;
-  if (cudaGetDevice(&dev) == cudaSuccess)
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  if ((long long)a.B * a.H * ((a.Nq + kBM - 1) / kBM) < 2LL * sms) {
-    const int n_qtiles = int((a.Nq + kSmallRows - 1) / kSmallRows);
-    const long long grid = (long long)a.B * a.H * n_qtiles;
-    if (grid > 0x7fffffffLL) {
-      snprintf(msg, msglen, "fp32 path: too many rows");
-      return 3;
-    }
-    const cudaError_t attr_err =
-        ensure_smem_limit(reinterpret_cast<const void*>(attn_fwd_f32_small_kernel),
-                          int(SmallSmem::bytes(kMaxD, kMaxD)));
-    if (attr_err != cudaSuccess) {
-      snprintf(msg, msglen, "cudaFuncSetAttribute (fp32 small kernel): %s",
-               cudaGetErrorString(attr_err));
-      return 5;
-    }
-    attn_fwd_f32_small_kernel<<<dim3(unsigned(grid)), dim3(kSmallThreads),
-                                SmallSmem::bytes(int(a.dk), int(a.dv)), a.stream>>>(
-        static_cast<const float*>(a.Q), static_cast<const float*>(a.K),
-        static_cast<const float*>(a.V), static_cast<float*>(a.O), a.lse, int(a.Nq), int(a.Nk),
-        int(a.dk), int(a.dv), n_qtiles, a.scale);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) {
-      snprintf(msg, msglen, "fp32 small kernel launch: %s", cudaGetErrorString(e));
-      return 5;
-    }
-    return 0;
-  }
-  const int n_qtiles = int((a.Nq + kBM - 1) / kBM);
+template <int VC, int R, int WR, int KW>
+int launch_tiled(const AttnArgs& a, char* msg, size_t msglen) {
+  using T = F32Tile<VC, R, WR, KW>;
+  const int n_qtiles = int((a.Nq + T::kBM - 1) / T::kBM);
   const long long grid = (long long)a.B * a.H * n_qtiles;
   if (grid > 0x7fffffffLL) {
-    snprintf(msg, msglen, "fp32 path: B*H*ceil(N_q/%d) = %lld CTAs exceeds the grid limit", kBM, grid);
+    snprintf(msg, msglen, "fp32 path: B*H*ceil(N_q/%d) = %lld CTAs exceeds the grid limit", T::kBM, grid);
     return 3;
   }
-  const size_t smem = F32Smem::bytes(int(a.dk), int(a.dv));
-  cudaError_t e = ensure_smem_limit(reinterpret_cast<const void*>(attn_fwd_f32_cc_kernel), int(smem));
+  auto kern = attn_fwd_f32_cc_kernel<VC, R, WR, KW>;
+  const size_t smem = T::smem_bytes(int(a.dk));
+  cudaError_t e = ensure_smem_limit(reinterpret_cast<const void*>(kern), int(smem));
   if (e != cudaSuccess) {
     snprintf(msg, msglen, "cudaFuncSetAttribute (fp32 kernel): %s", cudaGetErrorString(e));
     return 5;
   }
-  attn_fwd_f32_cc_kernel<<<dim3(unsigned(grid)), dim3(kThreads), smem, a.stream>>>(
+  kern<<<dim3(unsigned(grid)), dim3(T::kThreads), smem, a.stream>>>(
       static_cast<const float*>(a.Q), static_cast<const float*>(a.K),
       static_cast<const float*>(a.V), static_cast<float*>(a.O), a.lse, int(a.Nq), int(a.Nk),
       int(a.dk), int(a.dv), n_qtiles, a.scale);
@@ -392,6 +305,94 @@ int launch_attn_fwd_f32(const AttnArgs& a, char* msg, size_t msglen) {
     return 5;
   }
   return 0;
+}
+
+// The tile shapes, with the measured time of one step of a CTA (us at d = 64; the ratios hold for
+// other d): alone on its SM, and per CTA when `occ` of them share it.
+struct TileShape {
+  int r, wr, kw, occ;
+  float lone, shared;
+};
+constexpr TileShape kTiles[] = {
+    {8, 4, 2, 1, 14.0f, 14.0f}, {4, 4, 2, 2, 8.7f, 7.75f}, {4, 2, 2, 2, 5.6f, 4.3f},
+    {2, 2, 2, 2, 3.9f, 3.0f},   {1, 2, 2, 2, 3.0f, 2.4f},  {4, 2, 4, 1, 9.0f, 9.0f},
+    {4, 1, 4, 1, 6.4f, 6.4f},   {2, 1, 4, 1, 4.6f, 4.6f},  {1, 1, 4, 1, 4.0f, 4.0f}};
+constexpr float kRoundStart = 2.0f;  // first tiles of a CTA and the merge, same unit
+
+// Shared memory of a tile shape (F32Tile::smem_bytes with run-time sizes).
+size_t tile_smem(const TileShape& t, int dk, int vc) {
+  const size_t rows = 4 * size_t(t.r) * t.wr;
+  return sizeof(float) * (rows * odd_stride(dk) +
+                          size_t(kBN) * t.kw * (odd_stride(dk) + 32 * vc) + rows * t.kw * kLdp);
+}
+
+// Key groups, from the sizes of one (b, h) slice alone: the groups' merge decides the last bits of
+// a slice, which must not depend on how many slices a call has.  Four groups where a slice has few
+// rows (its calls are bound by the chain over the keys: 1x4x60x2000 64 -> 33 us, 1x32x300x700 83 ->
+// 80 us) and their tiles fit; two else (at N_q >= 512 larger row tiles do the same work in less:
+// 1x16x512x512 56 -> 39 us).
+int key_groups(const AttnArgs& a, int dk, int vc) {
+  return a.Nq < 512 && a.Nk > 2 * kBN && tile_smem({4, 2, 4, 1, 0, 0}, dk, vc) <= size_t(kMaxSmem) ? 4 : 2;
+}
+
+// The shape with the least estimated time: rounds of CTAs over the SMs x key steps x step time.
+int pick_tile(const AttnArgs& a, int sms) {
+  const int dk = int(a.dk), vc = int((a.dv + 31) / 32);
+  const int kw = key_groups(a, dk, vc);
+  int best = -1;
+  double best_time = 0;
+  for (int i = 0; i < int(sizeof(kTiles) / sizeof(kTiles[0])); ++i) {
+    const TileShape& t = kTiles[i];
+    const size_t smem = tile_smem(t, dk, vc);
+    if (t.kw != kw || smem > size_t(kMaxSmem)) continue;
+    // two CTAs an SM need the 128-register instances (d_v <= 64) and half the shared memory each
+    const int occ = t.occ == 2 && vc <= 2 && smem <= size_t(kMaxSmem + 1024) / 2 - 1024 ? 2 : 1;
+    const int64_t rows = 4 * t.r * t.wr, keys = int64_t(kBN) * t.kw;
+    const double n = double(a.B * a.H) * double((a.Nq + rows - 1) / rows);
+    const double steps = double((a.Nk + keys - 1) / keys);
+    const double slots = double(sms) * occ, full = floor(n / slots), rem = n - full * slots;
+    const double busy = occ * t.shared * steps + kRoundStart;
+    const double tail = rem <= 0 ? 0.0 : rem <= sms ? t.lone * steps + kRoundStart : busy;
+    const double time = full * busy + tail;
+    if (best < 0 || time < best_time) {
+      best = i;
+      best_time = time;
+    }
+  }
+  return best;
+}
+
+template <int VC>
+int launch_shape(int tile, const AttnArgs& a, char* msg, size_t msglen) {
+  switch (tile) {
+    case 0: return launch_tiled<VC, 8, 4, 2>(a, msg, msglen);
+    case 1: return launch_tiled<VC, 4, 4, 2>(a, msg, msglen);
+    case 2: return launch_tiled<VC, 4, 2, 2>(a, msg, msglen);
+    case 3: return launch_tiled<VC, 2, 2, 2>(a, msg, msglen);
+    case 4: return launch_tiled<VC, 1, 2, 2>(a, msg, msglen);
+    case 5: return launch_tiled<VC, 4, 2, 4>(a, msg, msglen);
+    case 6: return launch_tiled<VC, 4, 1, 4>(a, msg, msglen);
+    case 7: return launch_tiled<VC, 2, 1, 4>(a, msg, msglen);
+    case 8: return launch_tiled<VC, 1, 1, 4>(a, msg, msglen);
+  }
+  snprintf(msg, msglen, "fp32 path: no tile fits d_k=%lld d_v=%lld", (long long)a.dk, (long long)a.dv);
+  return 3;
+}
+
+}  // namespace
+
+int launch_attn_fwd_f32(const AttnArgs& a, char* msg, size_t msglen) {
+  int sms = 0;
+  const cudaError_t e = device_sm_count(&sms);
+  if (e != cudaSuccess) {
+    snprintf(msg, msglen, "fp32 path: SM count: %s", cudaGetErrorString(e));
+    return 5;
+  }
+  const int tile = pick_tile(a, sms);
+  if (a.dv <= 32) return launch_shape<1>(tile, a, msg, msglen);
+  if (a.dv <= 64) return launch_shape<2>(tile, a, msg, msglen);
+  if (a.dv <= 96) return launch_shape<3>(tile, a, msg, msglen);
+  return launch_shape<4>(tile, a, msg, msglen);
 }
 
 }  // namespace moa
