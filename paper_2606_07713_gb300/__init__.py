@@ -31,24 +31,54 @@ __all__ = ["attn_fwd", "attn_fwd_staged", "get_device_status", "attn_flops", "dn
            "moa_attn_bwd_fused", "moa_attn_bwd_fused_workspace_bytes"]
 
 
-def _dtype_code(t) -> int:
+_torch = None  # the torch module, bound by the first call (the package imports without torch)
+
+
+def _bind_torch():
+    global _torch
     import torch
-    if t.dtype == torch.bfloat16:
+    _torch = torch
+    return torch
+
+
+def _dtype_code(t) -> int:
+    torch = _torch or _bind_torch()
+    dt = t.dtype
+    if dt is torch.bfloat16:
         return MOA_BF16
-    if t.dtype == torch.float32:
+    if dt is torch.float32:
         return MOA_FP32
-    raise TypeError(f"unsupported dtype {t.dtype}; use torch.bfloat16 or torch.float32")
+    raise TypeError(f"unsupported dtype {dt}; use torch.bfloat16 or torch.float32")
 
 
 def _dims(q, k, v):
-    if q.dim() != 4 or k.dim() != 4 or v.dim() != 4:
+    qs, ks, vs = q.shape, k.shape, v.shape
+    if len(qs) != 4 or len(ks) != 4 or len(vs) != 4:
         raise ValueError("q, k, v must be [B, H, N, d]")
-    B, H, Nq, dk = q.shape
-    if tuple(k.shape[:2]) != (B, H) or tuple(v.shape[:2]) != (B, H):
-        raise ValueError(f"batch/head mismatch: {tuple(q.shape)} {tuple(k.shape)} {tuple(v.shape)}")
-    if k.shape[3] != dk or v.shape[2] != k.shape[2]:
-        raise ValueError(f"shape mismatch: {tuple(q.shape)} {tuple(k.shape)} {tuple(v.shape)}")
-    return B, H, Nq, k.shape[2], dk, v.shape[3]
+    B, H, Nq, dk = qs
+    kb, kh, Nk, kd = ks
+    vb, vh, vn, dv = vs
+    if kb != B or kh != H or vb != B or vh != H:
+        raise ValueError(f"batch/head mismatch: {tuple(qs)} {tuple(ks)} {tuple(vs)}")
+    if kd != dk or vn != Nk:
+        raise ValueError(f"shape mismatch: {tuple(qs)} {tuple(ks)} {tuple(vs)}")
+    return B, H, Nq, Nk, dk, dv
+
+
+def _call(fn, device, stream, *args) -> None:
+    """fn(*args, stream) on `device` (stream None: torch's current one); raises on a non-OK status.
+    A small call is bound by this host path: the raw stream handle and the current-device test take
+    0.3 us where a Stream object and a device guard took 3.6 us."""
+    torch = _torch or _bind_torch()
+    index = device.index
+    s = torch._C._cuda_getCurrentRawStream(index) if stream is None else stream.cuda_stream
+    if torch._C._cuda_getDevice() == index:
+        status = fn(*args, s)
+    else:
+        with torch.cuda.device(device):
+            status = fn(*args, s)
+    if status != 0:
+        check(status)
 
 
 def attn_fwd(q, k, v, scale: float | None = None, out=None, stream=None):
@@ -57,7 +87,6 @@ def attn_fwd(q, k, v, scale: float | None = None, out=None, stream=None):
     scale defaults to 1/sqrt(d_k).  Runs asynchronously on `stream` (default:
     torch's current stream of q's device) and returns `out` (allocated if None).
     """
-    import torch
     for t in (q, k, v):
         if not t.is_cuda:
             raise ValueError("attn_fwd needs CUDA tensors")
@@ -69,21 +98,19 @@ def attn_fwd(q, k, v, scale: float | None = None, out=None, stream=None):
     B, H, Nq, Nk, dk, dv = _dims(q, k, v)
     if scale is None:
         scale = 1.0 / math.sqrt(dk)
+    device = q.device
     if out is None:
-        out = torch.empty((B, H, Nq, dv), dtype=q.dtype, device=q.device)
+        out = _torch.empty((B, H, Nq, dv), dtype=q.dtype, device=device)
     elif out.shape != (B, H, Nq, dv) or out.dtype != q.dtype or not out.is_contiguous():
         raise ValueError("out has the wrong shape, dtype or layout")
-    with torch.cuda.device(q.device):
-        s = stream if stream is not None else torch.cuda.current_stream(q.device)
-        check(moa_attn_fwd(q.data_ptr(), k.data_ptr(), v.data_ptr(), out.data_ptr(), B, H, Nq, Nk,
-                           dk, dv, float(scale), code, s.cuda_stream))
+    _call(lib().moa_attn_fwd, device, stream, q.data_ptr(), k.data_ptr(), v.data_ptr(),
+          out.data_ptr(), B, H, Nq, Nk, dk, dv, float(scale), code)
     return out
 
 
 def attn_fwd_lse(q, k, v, scale: float | None = None, out=None, lse=None, stream=None):
     """(O, LSE): attn_fwd's output and the float32 [B, H, N_q] natural-log log-sum-exp of each
     row's scaled scores, ln sum_k exp(scale <q_i, k_k>)."""
-    import torch
     for t in (q, k, v):
         if not t.is_cuda or not t.is_contiguous():
             raise ValueError("attn_fwd_lse needs contiguous CUDA tensors")
@@ -93,19 +120,17 @@ def attn_fwd_lse(q, k, v, scale: float | None = None, out=None, lse=None, stream
     B, H, Nq, Nk, dk, dv = _dims(q, k, v)
     if scale is None:
         scale = 1.0 / math.sqrt(dk)
+    device = q.device
     if out is None:
-        out = torch.empty((B, H, Nq, dv), dtype=q.dtype, device=q.device)
+        out = _torch.empty((B, H, Nq, dv), dtype=q.dtype, device=device)
     elif out.shape != (B, H, Nq, dv) or out.dtype != q.dtype or not out.is_contiguous():
         raise ValueError("out has the wrong shape, dtype or layout")
     if lse is None:
-        lse = torch.empty((B, H, Nq), dtype=torch.float32, device=q.device)
-    elif lse.shape != (B, H, Nq) or lse.dtype != torch.float32 or not lse.is_contiguous():
+        lse = _torch.empty((B, H, Nq), dtype=_torch.float32, device=device)
+    elif lse.shape != (B, H, Nq) or lse.dtype != _torch.float32 or not lse.is_contiguous():
         raise ValueError("lse must be a contiguous float32 [B, H, N_q] tensor")
-    with torch.cuda.device(q.device):
-        s = stream if stream is not None else torch.cuda.current_stream(q.device)
-        check(moa_attn_fwd_lse(q.data_ptr(), k.data_ptr(), v.data_ptr(), out.data_ptr(),
-                               lse.data_ptr(), B, H, Nq, Nk, dk, dv, float(scale), code,
-                               s.cuda_stream))
+    _call(lib().moa_attn_fwd_lse, device, stream, q.data_ptr(), k.data_ptr(), v.data_ptr(),
+          out.data_ptr(), lse.data_ptr(), B, H, Nq, Nk, dk, dv, float(scale), code)
     return out, lse
 
 
@@ -115,7 +140,6 @@ def attn_bwd(q, k, v, o, lse, do, scale: float | None = None, workspace=None, st
     (attn_fwd_lse).  CUDA tensors [B, H, N, d]; lse float32 [B, H, N_q].  fused=True runs
     moa_attn_bwd_fused (bf16, d_k = d_v = 64; the key blocks' dQ tiles are added in fp32 by TMA
     reductions, in a run-dependent order)."""
-    import torch
     for t in (q, k, v, o, do, lse):
         if not t.is_cuda or not t.is_contiguous():
             raise ValueError("attn_bwd needs contiguous CUDA tensors")
@@ -125,31 +149,29 @@ def attn_bwd(q, k, v, o, lse, do, scale: float | None = None, workspace=None, st
     B, H, Nq, Nk, dk, dv = _dims(q, k, v)
     if tuple(o.shape) != (B, H, Nq, dv) or tuple(do.shape) != (B, H, Nq, dv):
         raise ValueError("o and do must be [B, H, N_q, d_v]")
-    if tuple(lse.shape) != (B, H, Nq) or lse.dtype != torch.float32:
+    if tuple(lse.shape) != (B, H, Nq) or lse.dtype != _torch.float32:
         raise ValueError("lse must be float32 [B, H, N_q]")
     if scale is None:
         scale = 1.0 / math.sqrt(dk)
-    dq = torch.empty_like(q)
-    dkk = torch.empty_like(k)
-    dvv = torch.empty_like(v)
-    wsb = moa_attn_bwd_fused_workspace_bytes if fused else moa_attn_bwd_workspace_bytes
-    call = moa_attn_bwd_fused if fused else moa_attn_bwd
-    need = wsb(B, H, Nq, Nk, dk, dv, code)
+    dq = _torch.empty_like(q)
+    dkk = _torch.empty_like(k)
+    dvv = _torch.empty_like(v)
+    L = lib()
+    wsb = L.moa_attn_bwd_fused_workspace_bytes if fused else L.moa_attn_bwd_workspace_bytes
+    fn = L.moa_attn_bwd_fused if fused else L.moa_attn_bwd
+    device = q.device
     if workspace is None:
-        workspace = torch.empty(max(need, 16), dtype=torch.uint8, device=q.device)
-    with torch.cuda.device(q.device):
-        s = stream if stream is not None else torch.cuda.current_stream(q.device)
-        check(call(q.data_ptr(), k.data_ptr(), v.data_ptr(), o.data_ptr(), do.data_ptr(),
-                   lse.data_ptr(), dq.data_ptr(), dkk.data_ptr(), dvv.data_ptr(), B, H, Nq, Nk, dk,
-                   dv, float(scale), code, workspace.data_ptr(), workspace.numel(),
-                   s.cuda_stream))
+        need = wsb(B, H, Nq, Nk, dk, dv, code)
+        workspace = _torch.empty(max(need, 16), dtype=_torch.uint8, device=device)
+    _call(fn, device, stream, q.data_ptr(), k.data_ptr(), v.data_ptr(), o.data_ptr(), do.data_ptr(),
+          lse.data_ptr(), dq.data_ptr(), dkk.data_ptr(), dvv.data_ptr(), B, H, Nq, Nk, dk, dv,
+          float(scale), code, workspace.data_ptr(), workspace.numel())
     return dq, dkk, dvv
 
 
 def qkv_proj(x, w, H: int, d_k: int, d_v: int, out=None, stream=None):
     """(Q, K, V) = (X W_Q, X W_K, X W_V) in head-major layout [B, H, N, d] from x [B, N, d_model]
     and w [d_model, 2*H*d_k + H*d_v] (W_Q | W_K | W_V), bf16 CUDA tensors."""
-    import torch
     for t in (x, w):
         if not t.is_cuda or not t.is_contiguous():
             raise ValueError("qkv_proj needs contiguous CUDA tensors")
@@ -161,15 +183,14 @@ def qkv_proj(x, w, H: int, d_k: int, d_v: int, out=None, stream=None):
     B, N, d = x.shape
     if tuple(w.shape) != (d, 2 * H * d_k + H * d_v):
         raise ValueError(f"w must be {(d, 2 * H * d_k + H * d_v)}, got {tuple(w.shape)}")
+    device, dtype = x.device, x.dtype
     if out is None:
-        out = (torch.empty((B, H, N, d_k), dtype=x.dtype, device=x.device),
-               torch.empty((B, H, N, d_k), dtype=x.dtype, device=x.device),
-               torch.empty((B, H, N, d_v), dtype=x.dtype, device=x.device))
+        out = (_torch.empty((B, H, N, d_k), dtype=dtype, device=device),
+               _torch.empty((B, H, N, d_k), dtype=dtype, device=device),
+               _torch.empty((B, H, N, d_v), dtype=dtype, device=device))
     q, k, v = out
-    with torch.cuda.device(x.device):
-        s = stream if stream is not None else torch.cuda.current_stream(x.device)
-        check(moa_qkv_proj(x.data_ptr(), w.data_ptr(), q.data_ptr(), k.data_ptr(), v.data_ptr(),
-                           B, N, d, H, d_k, d_v, code, s.cuda_stream))
+    _call(lib().moa_qkv_proj, device, stream, x.data_ptr(), w.data_ptr(), q.data_ptr(),
+          k.data_ptr(), v.data_ptr(), B, N, d, H, d_k, d_v, code)
     return q, k, v
 
 
@@ -181,7 +202,6 @@ def attn_fwd_splitkv(q, k, v, num_splits: int = MOA_SPLITS_AUTO, scale: float | 
     predicts a saving); otherwise nothing is split and the result is attn_fwd's.  The workspace
     (a CUDA uint8 tensor of at least moa_attn_splitkv_workspace_bytes(...) bytes) is allocated
     here when not given."""
-    import torch
     for t in (q, k, v):
         if not t.is_cuda or not t.is_contiguous():
             raise ValueError("attn_fwd_splitkv needs contiguous CUDA tensors")
@@ -191,16 +211,20 @@ def attn_fwd_splitkv(q, k, v, num_splits: int = MOA_SPLITS_AUTO, scale: float | 
     B, H, Nq, Nk, dk, dv = _dims(q, k, v)
     if scale is None:
         scale = 1.0 / math.sqrt(dk)
+    device = q.device
     if out is None:
-        out = torch.empty((B, H, Nq, dv), dtype=q.dtype, device=q.device)
-    with torch.cuda.device(q.device):
-        need = moa_attn_splitkv_workspace_bytes(B, H, Nq, Nk, dk, dv, code, int(num_splits))
-        if workspace is None:
-            workspace = torch.empty(max(need, 16), dtype=torch.uint8, device=q.device)
-        s = stream if stream is not None else torch.cuda.current_stream(q.device)
-        check(moa_attn_fwd_splitkv(q.data_ptr(), k.data_ptr(), v.data_ptr(), out.data_ptr(), B, H,
-                                   Nq, Nk, dk, dv, float(scale), code, int(num_splits),
-                                   workspace.data_ptr(), workspace.numel(), s.cuda_stream))
+        out = _torch.empty((B, H, Nq, dv), dtype=q.dtype, device=device)
+    L, splits = lib(), int(num_splits)
+    if workspace is None:
+        if _torch._C._cuda_getDevice() == device.index:
+            need = L.moa_attn_splitkv_workspace_bytes(B, H, Nq, Nk, dk, dv, code, splits)
+        else:  # MOA_SPLITS_AUTO reads the current device
+            with _torch.cuda.device(device):
+                need = L.moa_attn_splitkv_workspace_bytes(B, H, Nq, Nk, dk, dv, code, splits)
+        workspace = _torch.empty(max(need, 16), dtype=_torch.uint8, device=device)
+    _call(L.moa_attn_fwd_splitkv, device, stream, q.data_ptr(), k.data_ptr(), v.data_ptr(),
+          out.data_ptr(), B, H, Nq, Nk, dk, dv, float(scale), code, splits, workspace.data_ptr(),
+          workspace.numel())
     return out
 
 
@@ -208,7 +232,6 @@ def attn_fwd_staged(hq, hk, hv, ho, dq, dk_, dv_, do, scale: float | None = None
     """Host tensors in, host tensor out: copies hq/hk/hv to the device buffers dq/dk_/dv_,
     runs the kernel into do and copies it back into ho, all on one stream.  The result is in
     ho after the stream is synchronised."""
-    import torch
     code = _dtype_code(dq)
     B, H, Nq, Nk, dk, dv = _dims(dq, dk_, dv_)
     for h, d in ((hq, dq), (hk, dk_), (hv, dv_), (ho, do)):
@@ -218,11 +241,9 @@ def attn_fwd_staged(hq, hk, hv, ho, dq, dk_, dv_, do, scale: float | None = None
             raise ValueError("staged call needs contiguous tensors")
     if scale is None:
         scale = 1.0 / math.sqrt(dk)
-    with torch.cuda.device(dq.device):
-        s = stream if stream is not None else torch.cuda.current_stream(dq.device)
-        check(moa_attn_fwd_staged(hq.data_ptr(), hk.data_ptr(), hv.data_ptr(), ho.data_ptr(),
-                                  dq.data_ptr(), dk_.data_ptr(), dv_.data_ptr(), do.data_ptr(),
-                                  B, H, Nq, Nk, dk, dv, float(scale), code, s.cuda_stream))
+    _call(lib().moa_attn_fwd_staged, dq.device, stream, hq.data_ptr(), hk.data_ptr(), hv.data_ptr(),
+          ho.data_ptr(), dq.data_ptr(), dk_.data_ptr(), dv_.data_ptr(), do.data_ptr(), B, H, Nq, Nk,
+          dk, dv, float(scale), code)
     return ho
 
 
