@@ -28,9 +28,10 @@
 //   warp 9:    the single thread that issues all TMA loads;
 //   warp 10:   issues the tcgen05.mma products of Q tile 1;
 //   warp 11:   idle (it completes warps 8-11 as one warpgroup for the register split).
-// One-tile kernel (d_k = d_v = 64 without a split key axis; two CTAs per SM, 256 TMEM columns
-// and ~98 KB of shared memory each): work item = (b*H + h, block of 128 query rows); warps 0-3
-// softmax + epilogue, warp 4 TMEM allocation and tcgen05.mma, warp 5 TMA loads.
+// One-tile kernel (d_k = d_v = 64 without a split key axis, and every call of at most 128 query
+// rows): work item = (b*H + h, block of 128 query rows); warps 0-3 softmax + epilogue, warp 4 TMEM
+// allocation and tcgen05.mma, warp 5 TMA loads.  At d_k = d_v = 64 two CTAs share an SM (256 TMEM
+// columns and ~98 KB of shared memory each); otherwise one CTA with a 6-stage ring.
 // K and V tiles of 128 keys stream through an NS-stage shared-memory ring, in the order the
 // products use them: K0 K1 V0 K2 V1 ...  TMEM columns: S0 S1 P0 P1 O0 O1 at d_v = 64; one S
 // buffer shared by the two tiles, S P0 P1 O0 O1, at d_v = 128 (the two O take 256 columns);
@@ -77,12 +78,11 @@ template <int DK, int DV, int QT = 2>
 struct Cfg {
   static_assert(DK == 64 || DK == 128, "d_k must be 64 or 128");
   static_assert(QT == 1 || QT == 2, "one or two Q tiles per CTA");
-  static_assert(QT == 2 || DV == 64, "one-tile CTAs hold S, P and O of d_v = 64");
   // Warps: 4 softmax warps per Q tile, then the MMA warp of tile 0 (it also allocates and frees
-  // TMEM), the TMA warp and, with two tiles, the MMA warp of tile 1.  One-tile CTAs run two per
-  // SM (half the registers, TMEM and shared memory each).
+  // TMEM), the TMA warp and, with two tiles, the MMA warp of tile 1.  One-tile CTAs of d = 64 run
+  // two per SM (half the registers, TMEM and shared memory each).
   static constexpr int kThreads = QT == 2 ? 384 : 192;
-  static constexpr int kMinBlocks = QT == 2 ? 1 : 2;
+  static constexpr int kMinBlocks = QT == 1 && DK == 64 && DV == 64 ? 2 : 1;
   static constexpr int kMmaWarp0 = 4 * QT;
   static constexpr int kLoadWarp = 4 * QT + 1;
   static constexpr int kMmaWarp1 = QT == 2 ? 10 : -1;
@@ -98,7 +98,7 @@ struct Cfg {
   static constexpr int kRegsLaunch = 168, kRegsSoftmax = 208, kRegsCtrl = 88;
   static_assert(!kRegSplit || 256 * kRegsSoftmax + 128 * kRegsCtrl <= kThreads * kRegsLaunch,
                 "register split");
-  static constexpr int kTmemCols = 256 * QT;
+  static constexpr int kTmemCols = QT == 1 && DV == 64 ? 256 : 512;
   static_assert(DV == 64 || DV == 128, "d_v must be 64 or 128");
   // One 128-byte swizzle panel holds 64 bf16 columns of 128 rows: 16 KB.
   static constexpr int kPanelBytes = 128 * 128;
@@ -114,7 +114,7 @@ struct Cfg {
   // softmax holds its S(n).  (P in shared memory instead, with an S buffer per tile, measured
   // the same; it moves 128 KB more per key block through shared memory.)  One tile: S0 P0 O0.
   static constexpr bool kSharedS = QT == 2 && DV == 128;
-  static constexpr int kStages = QT == 1 ? (DK == 64 ? 5 : 2)
+  static constexpr int kStages = QT == 1 ? (kMinBlocks == 2 ? 5 : 6)
                                  : (DK == 64 && DV == 64) ? 8
                                  : kSharedS ? (DK == 128 ? 5 : 6) : 4;
   static constexpr int kOffQ = 0;
@@ -140,7 +140,7 @@ struct Cfg {
   static constexpr uint32_t kTmemO1 = kTmemO0 + DV;
   static_assert((QT == 2 ? kTmemO1 : kTmemO0) + DV <= kTmemCols, "TMEM budget");
   // Per SM: 228 KB, 1 KB of it reserved per CTA.
-  static_assert(kSmemBytes <= (QT == 2 ? 232448 : 233472 / 2 - 1024), "shared memory budget");
+  static_assert(kSmemBytes <= (kMinBlocks == 1 ? 232448 : 233472 / 2 - 1024), "shared memory budget");
 };
 
 // Maximum of 128 values (of their negations if NEG) with four independent 3-input chains.
@@ -187,7 +187,6 @@ attn_fwd_bf16_tc_kernel(const __grid_constant__ CUtensorMap tmQ,
                         int n_splits, int kv_per_split, float* __restrict__ ws_o,
                         float2* __restrict__ ws_ml, float* __restrict__ lse) {
   using C = Cfg<DK, DV, QT>;
-  static_assert(!SPLIT || QT == 2, "split key axes use two-tile CTAs");
   constexpr int kQTiles = QT;
   constexpr int kMmaWarp0 = C::kMmaWarp0, kLoadWarp = C::kLoadWarp, kMmaWarp1 = C::kMmaWarp1;
   constexpr int kTmemCols = C::kTmemCols;
@@ -254,6 +253,7 @@ attn_fwd_bf16_tc_kernel(const __grid_constant__ CUtensorMap tmQ,
   __syncthreads();
   tc_fence_after_sync();
   const uint32_t tmem = *tmem_slot;
+  if constexpr (SPLIT) launch_dependents();  // the merge kernel, which waits for this grid's end
 
   if (warp >= 4 * QT) {
     // Control warps (MMA issuers, TMA producer, and with two tiles an idle warp).
@@ -593,31 +593,57 @@ attn_fwd_bf16_tc_kernel(const __grid_constant__ CUtensorMap tmQ,
 // Merge of a split key axis (the identity behind Eq. stable_softmax applied across key ranges):
 // with per-split reference maxima m_s (log2 units), unnormalised rows O_s and sums l_s,
 //   M = max_s m_s,  O = sum_s 2^(m_s - M) O_s / sum_s 2^(m_s - M) l_s.
-// One warp per output row; lane c handles columns c, c+32, ...
+// One warp per output row, DV/32 neighbouring columns per lane.  The kernel is two round trips to L2
+// long: the (m, l) pairs of 32 splits come in one load (lane = split), then the rows of all splits.
+// (One pair at a time and strided 4-byte columns took 1.7 us more on 4096 rows x 9 splits.)
 template <int DV>
 __global__ void __launch_bounds__(256)
 splitkv_merge_kernel(const float* __restrict__ ws_o, const float2* __restrict__ ws_ml,
                      __nv_bfloat16* __restrict__ O, long long rows, int n_splits) {
+  constexpr int kCols = DV / 32;
   const long long r = (long long)blockIdx.x * 8 + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
+  grid_dependency_wait();  // launched while the split kernel ends: its partials are complete here
   if (r >= rows) return;
   float M = -INFINITY;
-  for (int s = 0; s < n_splits; ++s) M = fmaxf(M, ws_ml[s * rows + r].x);
+  for (int s0 = 0; s0 < n_splits; s0 += 32)
+    if (s0 + lane < n_splits) M = fmaxf(M, ws_ml[(s0 + lane) * rows + r].x);
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, off));
   float L = 0.f;
-  float acc[DV / 32];
+  float acc[kCols];
 #pragma unroll
-  for (int i = 0; i < DV / 32; ++i) acc[i] = 0.f;
-  for (int s = 0; s < n_splits; ++s) {
-    const float2 ml = ws_ml[s * rows + r];
-    const float w = ex2_approx(ml.x - M);
-    L = fmaf(w, ml.y, L);
-    const float* src = ws_o + (s * rows + r) * DV;
-#pragma unroll
-    for (int i = 0; i < DV / 32; ++i) acc[i] = fmaf(w, src[lane + 32 * i], acc[i]);
+  for (int i = 0; i < kCols; ++i) acc[i] = 0.f;
+  for (int s0 = 0; s0 < n_splits; s0 += 32) {
+    float w = 0.f, l = 0.f;
+    if (s0 + lane < n_splits) {
+      const float2 ml = ws_ml[(s0 + lane) * rows + r];
+      w = ex2_approx(ml.x - M);
+      l = ml.y;
+    }
+    const int n = min(32, n_splits - s0);
+#pragma unroll 4
+    for (int s = 0; s < n; ++s) {
+      const float ws = __shfl_sync(0xffffffffu, w, s), ls = __shfl_sync(0xffffffffu, l, s);
+      L = fmaf(ws, ls, L);
+      const float* src = ws_o + ((s0 + s) * rows + r) * DV + kCols * lane;
+      if constexpr (kCols == 4) {
+        const float4 v = *reinterpret_cast<const float4*>(src);
+        acc[0] = fmaf(ws, v.x, acc[0]);
+        acc[1] = fmaf(ws, v.y, acc[1]);
+        acc[2] = fmaf(ws, v.z, acc[2]);
+        acc[3] = fmaf(ws, v.w, acc[3]);
+      } else {
+        const float2 v = *reinterpret_cast<const float2*>(src);
+        acc[0] = fmaf(ws, v.x, acc[0]);
+        acc[1] = fmaf(ws, v.y, acc[1]);
+      }
+    }
   }
   const float inv = 1.0f / L;
+  uint32_t* dst = reinterpret_cast<uint32_t*>(O + r * DV + kCols * lane);
 #pragma unroll
-  for (int i = 0; i < DV / 32; ++i) O[r * DV + lane + 32 * i] = __float2bfloat16_rn(acc[i] * inv);
+  for (int i = 0; i < kCols; i += 2) dst[i >> 1] = pack_bf16x2(acc[i] * inv, acc[i + 1] * inv);
 }
 
 // Failure-path self test: one thread waits, with the kernel's bounded wait, on an mbarrier
@@ -724,32 +750,22 @@ namespace {
 template <int DK, int DV>
 constexpr bool kUseOneTile = DV == 64 && DK == 64;
 
-template <int DK, int DV>
-int launch_tc(const AttnArgs& a, const CUtensorMap& mq, const CUtensorMap& mk,
-              const CUtensorMap& mv, const SplitPlan& sp, void* ws, char* msg, size_t msglen) {
-  using C = Cfg<DK, DV>;
-  constexpr int QT1 = kUseOneTile<DK, DV> ? 1 : 2;
-  using C1 = Cfg<DK, DV, QT1>;
-  if (sp.n_splits > 1 && a.lse != nullptr) {
-    snprintf(msg, msglen, "the log-sum-exp output is not available with a split key axis");
-    return 1;
-  }
-  const bool split = sp.n_splits > 1;
-  auto kern = split ? attn_fwd_bf16_tc_kernel<DK, DV, true, 2>
-                    : attn_fwd_bf16_tc_kernel<DK, DV, false, QT1>;
-  const int threads = split ? C::kThreads : C1::kThreads;
-  const int smem_bytes = split ? C::kSmemBytes : C1::kSmemBytes;
-  const int tile_rows = split ? kQTiles * kBM : QT1 * kBM;
-  const cudaError_t attr_err = ensure_smem_limit(reinterpret_cast<const void*>(kern), smem_bytes);
+// One instance of the kernel: its shared-memory limit, the register-split check and the launch.
+template <int DK, int DV, bool SPLIT, int QT>
+int launch_instance(const AttnArgs& a, const CUtensorMap& mq, const CUtensorMap& mk,
+                    const CUtensorMap& mv, const SplitPlan& sp, float* ws_o, float2* ws_ml, char* msg,
+                    size_t msglen) {
+  using C = Cfg<DK, DV, QT>;
+  auto kern = attn_fwd_bf16_tc_kernel<DK, DV, SPLIT, QT>;
+  const cudaError_t attr_err = ensure_smem_limit(reinterpret_cast<const void*>(kern), C::kSmemBytes);
   if (attr_err != cudaSuccess) {
     snprintf(msg, msglen, "cudaFuncSetAttribute (bf16 kernel): %s", cudaGetErrorString(attr_err));
     return 5;
   }
-  if (split || QT1 == 2) {
+  if (C::kRegSplit) {
     // The register split of the two-tile kernel moves registers inside the CTA's launch
     // allocation: refuse a build whose allocation is short of the split's sum.
-    static std::atomic<int> regs_of[2] = {-1, -1};  // unsplit and split instance
-    std::atomic<int>& regs = regs_of[split ? 1 : 0];
+    static std::atomic<int> regs = {-1};
     if (regs.load(std::memory_order_relaxed) < 0) {
       cudaFuncAttributes fa;
       const cudaError_t e = cudaFuncGetAttributes(&fa, reinterpret_cast<const void*>(kern));
@@ -766,35 +782,57 @@ int launch_tc(const AttnArgs& a, const CUtensorMap& mq, const CUtensorMap& mk,
       return 5;
     }
   }
-  const int64_t n_qblocks = (a.Nq + tile_rows - 1) / tile_rows;
+  const int64_t n_qblocks = (a.Nq + QT * kBM - 1) / (QT * kBM);
   const int64_t grid = a.B * a.H * n_qblocks * sp.n_splits;
   if (grid > 0x7fffffffLL) {
     snprintf(msg, msglen, "bf16 path: %lld CTAs exceeds the grid limit", (long long)grid);
     return 3;
   }
   const float c_log2 = a.scale * 1.4426950408889634f;
-  const int64_t rows = a.B * a.H * a.Nq;
-  float* ws_o = sp.n_splits > 1 ? static_cast<float*>(ws) : nullptr;
-  float2* ws_ml = sp.n_splits > 1
-                      ? reinterpret_cast<float2*>(static_cast<float*>(ws) + sp.n_splits * rows * DV)
-                      : nullptr;
-  kern<<<dim3(unsigned(grid)), dim3(threads), smem_bytes, a.stream>>>(
+  kern<<<dim3(unsigned(grid)), dim3(C::kThreads), C::kSmemBytes, a.stream>>>(
       mq, mk, mv, static_cast<__nv_bfloat16*>(a.O), int(a.Nq), int(a.Nk), int(n_qblocks), c_log2,
       wait_limit_ns(), sp.n_splits, sp.kv_per_split, ws_o, ws_ml, a.lse);
-  cudaError_t e = cudaGetLastError();
+  const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) {
     snprintf(msg, msglen, "bf16 kernel launch: %s", cudaGetErrorString(e));
     return 5;
   }
-  if (sp.n_splits > 1) {
-    const long long blocks = (rows + 7) / 8;
-    splitkv_merge_kernel<DV><<<dim3(unsigned(blocks)), dim3(256), 0, a.stream>>>(
-        ws_o, ws_ml, static_cast<__nv_bfloat16*>(a.O), rows, sp.n_splits);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) {
-      snprintf(msg, msglen, "split merge launch: %s", cudaGetErrorString(e));
-      return 5;
-    }
+  return 0;
+}
+
+// At most 128 query rows fill one Q tile: a second tile's products and exponentials would be spent
+// on rows that do not exist, and they, not the loads of K and V, would set the pace of a key block.
+// Two-tile -> one-tile CTAs on a GB300: 8x16x1x8191 d=128 94.7 -> 79.7 us (6.7 TB/s of K and V),
+// 1x4x4x60000 d=128 (22 splits) 47.1 -> 36.5 us, 2x40x3x9000 d=64 (3 splits) 73.4 -> 39.7 us,
+// 1x32x128x16384 d=64 (4 splits) 50.4 -> 41.3 us.  From 129 rows on both tiles have rows.
+template <int DK, int DV>
+int launch_tc(const AttnArgs& a, const CUtensorMap& mq, const CUtensorMap& mk,
+              const CUtensorMap& mv, const SplitPlan& sp, void* ws, char* msg, size_t msglen) {
+  if (sp.n_splits > 1 && a.lse != nullptr) {
+    snprintf(msg, msglen, "the log-sum-exp output is not available with a split key axis");
+    return 1;
+  }
+  const bool one = a.Nq <= kBM;
+  if (sp.n_splits <= 1) {
+    if (one || kUseOneTile<DK, DV>)
+      return launch_instance<DK, DV, false, 1>(a, mq, mk, mv, sp, nullptr, nullptr, msg, msglen);
+    if constexpr (!kUseOneTile<DK, DV>)
+      return launch_instance<DK, DV, false, 2>(a, mq, mk, mv, sp, nullptr, nullptr, msg, msglen);
+  }
+  const int64_t rows = a.B * a.H * a.Nq;
+  float* ws_o = static_cast<float*>(ws);
+  float2* ws_ml = reinterpret_cast<float2*>(ws_o + sp.n_splits * rows * DV);
+  const int rc = one ? launch_instance<DK, DV, true, 1>(a, mq, mk, mv, sp, ws_o, ws_ml, msg, msglen)
+                     : launch_instance<DK, DV, true, 2>(a, mq, mk, mv, sp, ws_o, ws_ml, msg, msglen);
+  if (rc != 0) return rc;
+  const long long blocks = (rows + 7) / 8;
+  const cudaError_t e = launch_dependent(splitkv_merge_kernel<DV>, dim3(unsigned(blocks)), dim3(256), 0,
+                                         a.stream, static_cast<const float*>(ws_o),
+                                         static_cast<const float2*>(ws_ml),
+                                         static_cast<__nv_bfloat16*>(a.O), rows, sp.n_splits);
+  if (e != cudaSuccess) {
+    snprintf(msg, msglen, "split merge launch: %s", cudaGetErrorString(e));
+    return 5;
   }
   return 0;
 }

@@ -48,6 +48,24 @@ cudaError_t device_sm_count(int* sms);
 // per device, so the call is made once per (kernel, device, size) and its result remembered.
 cudaError_t ensure_smem_limit(const void* func, int bytes);
 
+// Launches a kernel that may start while the one before it on the stream is ending (programmatic
+// dependent launch); the kernel itself waits for that one's results.
+template <typename... Params, typename... Args>
+cudaError_t launch_dependent(void (*kern)(Params...), dim3 grid, dim3 block, size_t smem,
+                             cudaStream_t stream, Args... args) {
+  cudaLaunchConfig_t lc = {};
+  lc.gridDim = grid;
+  lc.blockDim = block;
+  lc.dynamicSmemBytes = smem;
+  lc.stream = stream;
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  lc.attrs = &attr;
+  lc.numAttrs = 1;
+  return cudaLaunchKernelEx(&lc, kern, args...);
+}
+
 // Size of the fixed device array behind the allocation-free split entry point (16 MiB).
 constexpr size_t kNoallocScratchBytes = size_t(16) << 20;
 
