@@ -160,6 +160,8 @@ attn_bwd_pre_kernel(const __nv_bfloat16* __restrict__ O, const __nv_bfloat16* __
   const int lane = threadIdx.x & 31;
   const long long r = ((long long)blockIdx.x * 8 + (threadIdx.x >> 5)) * kRows + lane / G;
   const int gl = lane % G;
+  launch_dependents();
+  grid_dependency_wait();
   const bool in_range = r < rows_pad;
   const long long bh = in_range ? r / Nq_pad : 0;
   const int i = in_range ? int(r % Nq_pad) : 0;
@@ -276,6 +278,10 @@ attn_bwd_dkdv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
   __syncthreads();
   tc_fence_after_sync();
   const uint32_t tmem = *tmem_slot;
+  // The per-row kernel has ended, here and, since the dQ kernel starts after this call in every CTA,
+  // there too: dQ CTAs take the SMs that the last round of this kernel leaves idle.
+  grid_dependency_wait();
+  launch_dependents();
 
   if (warp == kLoadWarp) {
     // ---------------------------------------------------------------- TMA producer
@@ -584,6 +590,7 @@ attn_bwd_dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
   __syncthreads();
   tc_fence_after_sync();
   const uint32_t tmem = *tmem_slot;
+  launch_dependents();  // (grid_dependency_wait is at the end: see the dK/dV kernel)
 
   if (warp == kLoadWarp) {
     // ---------------------------------------------------------------- TMA producer
@@ -706,7 +713,7 @@ attn_bwd_dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
     const uint32_t tS = tmem + lanes + C::kTmemS + part * kCols;
     const uint32_t tDP = tmem + lanes + C::kTmemDP + part * kCols;
     const size_t vrow = size_t(bh) * Nq_pad + size_t(q0 + row);  // padded: always in range
-    const float nl = nL[vrow], dd = Dd[vrow];
+    const float nl = __ldcg(nL + vrow), dd = __ldcg(Dd + vrow);
     const uint64_t cc = pack_f32x2(c_log2, c_log2);
     const uint64_t nn = pack_f32x2(nl, nl);
     bool ok = true;
@@ -759,6 +766,7 @@ attn_bwd_dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
     tc_fence_after_sync();
     tmem_dealloc(tmem, kTmemCols);
   }
+  grid_dependency_wait();  // this grid's end stands for the dK/dV kernel's too
 }
 
 
@@ -876,6 +884,8 @@ attn_bwd_fused_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
   __syncthreads();
   tc_fence_after_sync();
   const uint32_t tmem = *tmem_slot;
+  launch_dependents();     // what follows on the stream may take SMs as they come free
+  grid_dependency_wait();  // what came before has ended: its results are visible
 
   if (warp == C::kReduceWarp) {
     // ---------------------------------------------------------------- dQ reductions
@@ -1178,6 +1188,8 @@ __global__ void __launch_bounds__(256)
 attn_bwd_dq_convert_kernel(const float* __restrict__ dq_acc, __nv_bfloat16* __restrict__ dQ,
                            int Nq, int Nq_pad, long long n_items, float scale) {
   const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  launch_dependents();
+  grid_dependency_wait();
   if (t >= n_items) return;
   constexpr int kPerRow = DK / 8;
   const long long r = t / kPerRow;  // row of the real (unpadded) rows, head-major
@@ -1225,26 +1237,24 @@ int launch_bwd(const BwdArgs& a, const CUtensorMap& mq, const CUtensorMap& mk,
   const float c_log2 = a.scale * kLog2e;
   const long long rows_pad = BH * nq_pad;
   constexpr int kPreRowsPerBlock = 8 * (32 / (DV / 8));
-  attn_bwd_pre_kernel<DV><<<dim3(unsigned((rows_pad + kPreRowsPerBlock - 1) / kPreRowsPerBlock)),
-                            dim3(256), 0, a.stream>>>(
-      static_cast<const __nv_bfloat16*>(a.O), static_cast<const __nv_bfloat16*>(a.dO), a.lse, nL,
-      Dd, int(a.Nq), int(nq_pad), rows_pad);
-  cudaError_t e = cudaGetLastError();
+  cudaError_t e = launch_dependent(
+      attn_bwd_pre_kernel<DV>, dim3(unsigned((rows_pad + kPreRowsPerBlock - 1) / kPreRowsPerBlock)),
+      dim3(256), 0, a.stream, static_cast<const __nv_bfloat16*>(a.O),
+      static_cast<const __nv_bfloat16*>(a.dO), a.lse, nL, Dd, int(a.Nq), int(nq_pad), rows_pad,
+      static_cast<float*>(nullptr));
   if (e == cudaSuccess) {
-    attn_bwd_dkdv_kernel<DK, DV><<<dim3(unsigned(BH * n_kb)), dim3(A::kThreads), A::kSmemBytes,
-                                   a.stream>>>(
-        mq, mk, mv, mdo, nL, Dd, static_cast<__nv_bfloat16*>(a.dK),
-        static_cast<__nv_bfloat16*>(a.dV), int(a.Nk), int(nq_pad), int(n_kb), c_log2, a.scale,
-        wait_limit_ns());
-    e = cudaGetLastError();
+    e = launch_dependent(attn_bwd_dkdv_kernel<DK, DV>, dim3(unsigned(BH * n_kb)), dim3(A::kThreads),
+                         A::kSmemBytes, a.stream, mq, mk, mv, mdo, static_cast<const float*>(nL),
+                         static_cast<const float*>(Dd),
+                         static_cast<__nv_bfloat16*>(a.dK), static_cast<__nv_bfloat16*>(a.dV),
+                         int(a.Nk), int(nq_pad), int(n_kb), c_log2, a.scale, wait_limit_ns());
   }
   if (e == cudaSuccess) {
-    attn_bwd_dq_kernel<DK, DV><<<dim3(unsigned(BH * n_qb)), dim3(B::kThreads), B::kSmemBytes,
-                                 a.stream>>>(mq, mk, mv, mdo, nL, Dd,
-                                             static_cast<__nv_bfloat16*>(a.dQ), int(a.Nq),
-                                             int(a.Nk), int(nq_pad), int(n_qb), c_log2, a.scale,
-                                             wait_limit_ns());
-    e = cudaGetLastError();
+    e = launch_dependent(attn_bwd_dq_kernel<DK, DV>, dim3(unsigned(BH * n_qb)), dim3(B::kThreads),
+                         B::kSmemBytes, a.stream, mq, mk, mv, mdo, static_cast<const float*>(nL),
+                         static_cast<const float*>(Dd),
+                         static_cast<__nv_bfloat16*>(a.dQ), int(a.Nq), int(a.Nk), int(nq_pad),
+                         int(n_qb), c_log2, a.scale, wait_limit_ns());
   }
   if (e != cudaSuccess) {
     snprintf(msg, msglen, "bf16 backward launch: %s", cudaGetErrorString(e));
@@ -1280,24 +1290,21 @@ int launch_bwd_fused(const BwdArgs& a, const CUtensorMap& mq, const CUtensorMap&
   if (!encode_f32_map_sw128(&mdq, dq_acc, BH, nq_pad, DK, 32, kBlk, msg, msglen)) return 5;
   const float c_log2 = a.scale * kLog2e;
   constexpr int kPreRowsPerBlock = 8 * (32 / (DV / 8));
-  attn_bwd_pre_kernel<DV, DK><<<dim3(unsigned((rows_pad + kPreRowsPerBlock - 1) / kPreRowsPerBlock)),
-                                dim3(256), 0, a.stream>>>(
-      static_cast<const __nv_bfloat16*>(a.O), static_cast<const __nv_bfloat16*>(a.dO), a.lse, nL,
-      Dd, int(a.Nq), int(nq_pad), rows_pad, dq_acc);
-  cudaError_t e = cudaGetLastError();
+  cudaError_t e = launch_dependent(
+      attn_bwd_pre_kernel<DV, DK>, dim3(unsigned((rows_pad + kPreRowsPerBlock - 1) / kPreRowsPerBlock)),
+      dim3(256), 0, a.stream, static_cast<const __nv_bfloat16*>(a.O),
+      static_cast<const __nv_bfloat16*>(a.dO), a.lse, nL, Dd, int(a.Nq), int(nq_pad), rows_pad, dq_acc);
   if (e == cudaSuccess) {
-    attn_bwd_fused_kernel<DK, DV><<<dim3(unsigned(BH * n_kb)), dim3(F::kThreads), F::kSmemBytes,
-                                    a.stream>>>(
-        mq, mk, mv, mdo, mdq, nL, Dd, static_cast<__nv_bfloat16*>(a.dK),
-        static_cast<__nv_bfloat16*>(a.dV), int(a.Nk), int(nq_pad), int(n_kb), c_log2, a.scale,
-        wait_limit_ns());
-    e = cudaGetLastError();
+    e = launch_dependent(attn_bwd_fused_kernel<DK, DV>, dim3(unsigned(BH * n_kb)), dim3(F::kThreads),
+                         F::kSmemBytes, a.stream, mq, mk, mv, mdo, mdq, static_cast<const float*>(nL),
+                         static_cast<const float*>(Dd),
+                         static_cast<__nv_bfloat16*>(a.dK), static_cast<__nv_bfloat16*>(a.dV),
+                         int(a.Nk), int(nq_pad), int(n_kb), c_log2, a.scale, wait_limit_ns());
   }
   if (e == cudaSuccess) {
-    attn_bwd_dq_convert_kernel<DK><<<dim3(unsigned((n_conv + 255) / 256)), dim3(256), 0,
-                                     a.stream>>>(dq_acc, static_cast<__nv_bfloat16*>(a.dQ),
-                                                 int(a.Nq), int(nq_pad), n_conv, a.scale);
-    e = cudaGetLastError();
+    e = launch_dependent(attn_bwd_dq_convert_kernel<DK>, dim3(unsigned((n_conv + 255) / 256)), dim3(256),
+                         0, a.stream, static_cast<const float*>(dq_acc),
+                         static_cast<__nv_bfloat16*>(a.dQ), int(a.Nq), int(nq_pad), n_conv, a.scale);
   }
   if (e != cudaSuccess) {
     snprintf(msg, msglen, "fused backward launch: %s", cudaGetErrorString(e));

@@ -25,11 +25,14 @@
 
 #include "f32_common.cuh"
 #include "internal.h"
+#include "ptx.cuh"
 
 namespace moa {
 namespace {
 
 using namespace f32;
+using ptx::grid_dependency_wait;
+using ptx::launch_dependents;
 
 constexpr int kBN = 64;          // rows of the streamed axis per group and step
 constexpr int kHalf = kBN / 2;   // columns of P or dS held in shared memory at a time
@@ -64,6 +67,8 @@ attn_bwd_f32_pre_kernel(const float* __restrict__ O, const float* __restrict__ d
                         float* __restrict__ Dw, int Nq, int Nq_pad, int dv, long long rows) {
   const long long t = (long long)blockIdx.x * 8 + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
+  launch_dependents();
+  grid_dependency_wait();
   if (t >= rows) return;
   const long long bh = t / Nq;
   const int i = int(t % Nq);
@@ -318,6 +323,8 @@ attn_bwd_f32_kernel(const float* __restrict__ Q, const float* __restrict__ K,
                     float scale) {
   extern __shared__ __align__(16) float smem[];
   constexpr int kBM = BwdTile<C, R, WR, KW>::kBM;
+  launch_dependents();
+  grid_dependency_wait();
   if (blockIdx.x < n_dkdv) {
     const long long bh = blockIdx.x / n_ktiles;
     const long long k0 = (long long)(blockIdx.x % n_ktiles) * kBM;
@@ -345,12 +352,12 @@ cudaError_t launch_rows(const BwdArgs& a, const float* Lw, const float* Dw, int6
   auto kern = attn_bwd_f32_kernel<C, R, WR, KW>;
   const cudaError_t e = ensure_smem_limit(reinterpret_cast<const void*>(kern), int(smem));
   if (e != cudaSuccess) return e;
-  kern<<<dim3(unsigned(BH * (n_kt + n_qt))), dim3(T::kThreads), smem, a.stream>>>(
+  return launch_dependent(
+      kern, dim3(unsigned(BH * (n_kt + n_qt))), dim3(T::kThreads), smem, a.stream,
       static_cast<const float*>(a.Q), static_cast<const float*>(a.K),
       static_cast<const float*>(a.V), static_cast<const float*>(a.dO), Lw, Dw,
       static_cast<float*>(a.dQ), static_cast<float*>(a.dK), static_cast<float*>(a.dV), int(a.Nq),
       int(a.Nk), int(nq_pad), int(a.dk), int(a.dv), unsigned(BH * n_kt), int(n_kt), int(n_qt), a.scale);
-  return cudaGetLastError();
 }
 
 // The shape with the least estimated time: all CTAs' steps spread over the SMs plus half of the
@@ -412,10 +419,9 @@ int launch_attn_bwd_f32(const BwdArgs& a, char* msg, size_t msglen) {
   float* Lw = static_cast<float*>(a.ws);
   float* Dw = Lw + BH * nq_pad;
   const long long rows = BH * a.Nq;
-  attn_bwd_f32_pre_kernel<<<dim3(unsigned((rows + 7) / 8)), dim3(256), 0, a.stream>>>(
-      static_cast<const float*>(a.O), static_cast<const float*>(a.dO), a.lse, Lw, Dw,
-      int(a.Nq), int(nq_pad), dv, rows);
-  e = cudaGetLastError();
+  e = launch_dependent(attn_bwd_f32_pre_kernel, dim3(unsigned((rows + 7) / 8)), dim3(256), 0, a.stream,
+                       static_cast<const float*>(a.O), static_cast<const float*>(a.dO), a.lse, Lw, Dw,
+                       int(a.Nq), int(nq_pad), dv, rows);
   if (e == cudaSuccess) {
     const int d = dk > dv ? dk : dv;
     e = d <= 32 ? launch_shape<1>(tile, a, Lw, Dw, nq_pad)

@@ -253,7 +253,8 @@ attn_fwd_bf16_tc_kernel(const __grid_constant__ CUtensorMap tmQ,
   __syncthreads();
   tc_fence_after_sync();
   const uint32_t tmem = *tmem_slot;
-  if constexpr (SPLIT) launch_dependents();  // the merge kernel, which waits for this grid's end
+  launch_dependents();      // what follows on the stream may take SMs as they come free
+  grid_dependency_wait();   // what came before has ended: its results are visible
 
   if (warp >= 4 * QT) {
     // Control warps (MMA issuers, TMA producer, and with two tiles an idle warp).
@@ -603,6 +604,7 @@ splitkv_merge_kernel(const float* __restrict__ ws_o, const float2* __restrict__ 
   constexpr int kCols = DV / 32;
   const long long r = (long long)blockIdx.x * 8 + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
+  launch_dependents();
   grid_dependency_wait();  // launched while the split kernel ends: its partials are complete here
   if (r >= rows) return;
   float M = -INFINITY;
@@ -789,10 +791,10 @@ int launch_instance(const AttnArgs& a, const CUtensorMap& mq, const CUtensorMap&
     return 3;
   }
   const float c_log2 = a.scale * 1.4426950408889634f;
-  kern<<<dim3(unsigned(grid)), dim3(C::kThreads), C::kSmemBytes, a.stream>>>(
-      mq, mk, mv, static_cast<__nv_bfloat16*>(a.O), int(a.Nq), int(a.Nk), int(n_qblocks), c_log2,
+  const cudaError_t e = launch_dependent(
+      kern, dim3(unsigned(grid)), dim3(C::kThreads), C::kSmemBytes, a.stream, mq, mk, mv,
+      static_cast<__nv_bfloat16*>(a.O), int(a.Nq), int(a.Nk), int(n_qblocks), c_log2,
       wait_limit_ns(), sp.n_splits, sp.kv_per_split, ws_o, ws_ml, a.lse);
-  const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) {
     snprintf(msg, msglen, "bf16 kernel launch: %s", cudaGetErrorString(e));
     return 5;

@@ -35,11 +35,14 @@
 
 #include "f32_common.cuh"
 #include "internal.h"
+#include "ptx.cuh"
 
 namespace moa {
 namespace {
 
 using namespace f32;
+using ptx::grid_dependency_wait;
+using ptx::launch_dependents;
 
 constexpr int kBN = 64;                     // keys per key group and step
 constexpr int kHalf = kBN / 2;              // keys of P held in shared memory at a time
@@ -104,6 +107,8 @@ attn_fwd_f32_cc_kernel(const float* __restrict__ Q, const float* __restrict__ K,
         *reinterpret_cast<float4*>(dst + (r - row0) * ld) = make_float4(0.f, 0.f, 0.f, 0.f);
     }
   };
+  launch_dependents();
+  grid_dependency_wait();
   request(sQ, ldk, Qh, dk, q0, kBM, Nq);
   request(sK, ldk, Kh, dk, 0, kStep, Nk);
   cp_async_commit();
@@ -295,11 +300,10 @@ int launch_tiled(const AttnArgs& a, char* msg, size_t msglen) {
     snprintf(msg, msglen, "cudaFuncSetAttribute (fp32 kernel): %s", cudaGetErrorString(e));
     return 5;
   }
-  kern<<<dim3(unsigned(grid)), dim3(T::kThreads), smem, a.stream>>>(
-      static_cast<const float*>(a.Q), static_cast<const float*>(a.K),
-      static_cast<const float*>(a.V), static_cast<float*>(a.O), a.lse, int(a.Nq), int(a.Nk),
-      int(a.dk), int(a.dv), n_qtiles, a.scale);
-  e = cudaGetLastError();
+  e = launch_dependent(kern, dim3(unsigned(grid)), dim3(T::kThreads), smem, a.stream,
+                       static_cast<const float*>(a.Q), static_cast<const float*>(a.K),
+                       static_cast<const float*>(a.V), static_cast<float*>(a.O), a.lse, int(a.Nq),
+                       int(a.Nk), int(a.dk), int(a.dv), n_qtiles, a.scale);
   if (e != cudaSuccess) {
     snprintf(msg, msglen, "fp32 kernel launch: %s", cudaGetErrorString(e));
     return 5;

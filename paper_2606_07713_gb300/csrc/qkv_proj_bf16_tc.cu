@@ -144,6 +144,8 @@ qkv_proj_bf16_tc_kernel(const __grid_constant__ CUtensorMap tmX,
   cluster_sync();  // both CTAs' barriers are initialised before either is signalled
   tc_fence_after_sync();
   const uint32_t tmem = *tmem_slot;
+  launch_dependents();     // what follows on the stream may take SMs as they come free
+  grid_dependency_wait();  // what came before has ended: its results are visible
 
   if (warp == kLoadWarp) {
     if (lane == 0) {
@@ -382,6 +384,8 @@ qkv_proj_small_kernel(const __grid_constant__ CUtensorMap tmX,
   __syncthreads();
   tc_fence_after_sync();
   const uint32_t tmem = *tmem_slot;
+  launch_dependents();     // what follows on the stream may take SMs as they come free
+  grid_dependency_wait();  // what came before has ended: its results are visible
 
   if (warp == 0) {
     if (lane == 0) {
@@ -538,11 +542,13 @@ int launch_qkv_proj_bf16(const ProjArgs& a, char* msg, size_t msglen) {
     lc.blockDim = dim3(kSmallThreads);
     lc.dynamicSmemBytes = small_smem_bytes(sc);
     lc.stream = a.stream;
-    cudaLaunchAttribute attr;
-    attr.id = cudaLaunchAttributeClusterDimension;
-    attr.val.clusterDim = {unsigned(sc.ks), 1, 1};
-    lc.attrs = &attr;
-    lc.numAttrs = 1;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim = {unsigned(sc.ks), 1, 1};
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    lc.attrs = attr;
+    lc.numAttrs = 2;
     const cudaError_t e = cudaLaunchKernelEx(&lc, qkv_proj_small_kernel, mx, mw,
                                              static_cast<__nv_bfloat16*>(a.Q),
                                              static_cast<__nv_bfloat16*>(a.K),
@@ -563,10 +569,10 @@ int launch_qkv_proj_bf16(const ProjArgs& a, char* msg, size_t msglen) {
   p.n_whole = int(2 * rest <= pairs ? n_tiles - rest : n_tiles);
   p.n_items = int(p.n_whole + 2 * (n_tiles - p.n_whole));
   const int grid = 2 * int(p.n_items < pairs ? p.n_items : pairs);
-  qkv_proj_bf16_tc_kernel<<<dim3(unsigned(grid)), dim3(kThreads), kSmemBytes, a.stream>>>(
-      mx, mw, static_cast<__nv_bfloat16*>(a.Q), static_cast<__nv_bfloat16*>(a.K),
+  const cudaError_t e = launch_dependent(
+      qkv_proj_bf16_tc_kernel, dim3(unsigned(grid)), dim3(kThreads), kSmemBytes, a.stream, mx, mw,
+      static_cast<__nv_bfloat16*>(a.Q), static_cast<__nv_bfloat16*>(a.K),
       static_cast<__nv_bfloat16*>(a.V), p, wait_limit_ns());
-  cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) {
     snprintf(msg, msglen, "projection launch: %s", cudaGetErrorString(e));
     return 5;
