@@ -9,7 +9,7 @@
 // weights are rebuilt tile by tile from the scores and the forward pass's per-row log-sum-exp,
 // W_ik = exp2(c * s_ik - LSE_i * log2 e), c = scale * log2 e.
 //
-// Three kernels:
+// Three kernels, the second and third in either order and overlapping at their ends:
 //   attn_bwd_pre_kernel   per query row: D_i and -LSE_i * log2 e into a padded fp32 workspace
 //                         (rows past N_q get D = 0 and -inf, so padded queries weigh nothing);
 //   attn_bwd_dkdv_kernel  one CTA per (b, h, block of 128 keys); streams every 128-row query
@@ -18,7 +18,8 @@
 //                           P^T = exp2(c S^T - L), dS^T = P^T (dP^T - D)   (registers, per key row)
 //                           dV += P^T dO,  dK += dS^T Q           (A operand from TMEM, bf16)
 //   attn_bwd_dq_kernel    one CTA per (b, h, block of 128 query rows); streams the key blocks:
-//                           S = Q K^T, dP = dO V^T, dS = P (dP - D), dQ += dS K.
+//                           S = Q K^T, dP = dO V^T, dS = P (dP - D), dQ += dS K;
+//   attn_bwd_dq2_kernel   the same with 256 query rows per CTA, where the grid fills the GPU.
 // Splitting dQ from dK/dV keeps every accumulation inside one CTA (no atomics, deterministic
 // results) at the price of computing S and dP twice: 7 tile products per (query, key) block
 // pair instead of 5.
@@ -37,6 +38,7 @@
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
+#include <atomic>
 #include <cmath>
 #include <cstdio>
 
@@ -142,6 +144,19 @@ __device__ __forceinline__ void store_row_bf16(uint32_t taddr, float mul, __nv_b
   }
 }
 
+// The dK/dV and dQ kernels depend on the per-row kernel, not on each other, and the second of the two
+// launched takes the SMs that the first one's last round leaves idle.  The first waits for the per-row
+// kernel before it lets dependents start; so the second needs no wait of its own (it reads the per-row
+// values through L2).  Its end has to stand for the first one's too: one CTA of it, the last, ends
+// only after that grid (all of them waiting would hold SMs idle until then).
+__device__ __forceinline__ void tile_kernel_begin(bool second) {
+  if (!second) grid_dependency_wait();
+  launch_dependents();
+}
+__device__ __forceinline__ void tile_kernel_end(bool second) {
+  if (second && blockIdx.x == gridDim.x - 1) grid_dependency_wait();
+}
+
 // ------------------------------------------------------------------------------------------
 // Per-row preprocessing
 // ------------------------------------------------------------------------------------------
@@ -230,7 +245,8 @@ attn_bwd_dkdv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
                      const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmDO,
                      const float* __restrict__ nL, const float* __restrict__ Dd,
                      __nv_bfloat16* __restrict__ dK, __nv_bfloat16* __restrict__ dV, int Nk,
-                     int Nq_pad, int n_kblocks, float c_log2, float scale, uint64_t wait_limit_ns) {
+                     int Nq_pad, int n_kblocks, float c_log2, float scale, bool second,
+                     uint64_t wait_limit_ns) {
   using C = DkDvCfg<DK, DV>;
   constexpr int kParts = C::kParts, kCols = C::kCols, kComputeThreads = C::kComputeThreads;
   constexpr int kMmaWarp = C::kMmaWarp, kLoadWarp = C::kLoadWarp;
@@ -278,10 +294,7 @@ attn_bwd_dkdv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
   __syncthreads();
   tc_fence_after_sync();
   const uint32_t tmem = *tmem_slot;
-  // The per-row kernel has ended, here and, since the dQ kernel starts after this call in every CTA,
-  // there too: dQ CTAs take the SMs that the last round of this kernel leaves idle.
-  grid_dependency_wait();
-  launch_dependents();
+  tile_kernel_begin(second);
 
   if (warp == kLoadWarp) {
     // ---------------------------------------------------------------- TMA producer
@@ -509,6 +522,7 @@ attn_bwd_dkdv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
     tc_fence_after_sync();
     tmem_dealloc(tmem, kTmemCols);
   }
+  tile_kernel_end(second);
 }
 
 // ------------------------------------------------------------------------------------------
@@ -542,7 +556,7 @@ attn_bwd_dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
                    const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmDO,
                    const float* __restrict__ nL, const float* __restrict__ Dd,
                    __nv_bfloat16* __restrict__ dQ, int Nq, int Nk, int Nq_pad, int n_qblocks,
-                   float c_log2, float scale, uint64_t wait_limit_ns) {
+                   float c_log2, float scale, bool second, uint64_t wait_limit_ns) {
   using C = DqCfg<DK, DV>;
   constexpr int kCols = C::kCols, kComputeThreads = C::kComputeThreads;
   constexpr int kMmaWarp = C::kMmaWarp, kLoadWarp = C::kLoadWarp;
@@ -590,7 +604,7 @@ attn_bwd_dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
   __syncthreads();
   tc_fence_after_sync();
   const uint32_t tmem = *tmem_slot;
-  launch_dependents();  // (grid_dependency_wait is at the end: see the dK/dV kernel)
+  tile_kernel_begin(second);
 
   if (warp == kLoadWarp) {
     // ---------------------------------------------------------------- TMA producer
@@ -766,7 +780,320 @@ attn_bwd_dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
     tc_fence_after_sync();
     tmem_dealloc(tmem, kTmemCols);
   }
-  grid_dependency_wait();  // this grid's end stands for the dK/dV kernel's too
+  tile_kernel_end(second);
+}
+
+
+// ------------------------------------------------------------------------------------------
+// dQ, two query tiles per CTA: one CTA per (b, h, 256-row query block)
+// ------------------------------------------------------------------------------------------
+// The one-tile kernel's chain per key block (S, exponentials, dP, dS, dQ) leaves the tensor pipe idle
+// half of the time.  Here two 128-row tiles take turns, each with its own issuing thread and its own
+// warpgroup (one thread per query row), so that one tile's products run during the other's
+// exponentials.  To fit two tiles in tensor memory, S and dP of a tile share 128 columns X: the scores
+// leave for registers, where P stays in fp32, before dP arrives, and dS (bf16) is packed over dP's
+// first half as it is read:
+//   per tile and key block: S = Q K^T -> X | P = exp2(c S - L) in registers, dP = dO V^T -> X meanwhile
+//   | dS = P (dP - D) -> X | dQ += dS K.
+// TMEM: X0 X1 dQ0 dQ1.  K and V have rings of their own: K(n) is held from S(n) to dQ(n) of both
+// tiles, V(n) only while the two dP(n) run.  Warps: 0-3 and 4-7 compute tiles 0 and 1, 8 and 10 issue
+// their products, 9 TMA, 11 idle; registers move to the compute warps as in the forward kernel.
+template <int DK, int DV>
+struct Dq2Cfg {
+  static constexpr int kThreads = 384;
+  static constexpr int kMmaWarp0 = 8, kLoadWarp = 9, kMmaWarp1 = 10;
+  static constexpr int kRegsLaunch = 168, kRegsCompute = 208, kRegsCtrl = 88;
+  static_assert(256 * kRegsCompute + 128 * kRegsCtrl <= kThreads * kRegsLaunch, "register split");
+  static constexpr int kQBytes = kBlk * DK * 2, kDOBytes = kBlk * DV * 2;
+  static constexpr int kKBytes = kBlk * DK * 2, kVBytes = kBlk * DV * 2;
+  static constexpr int kKStages = DK == 128 ? 2 : 3;
+  static constexpr int kVStages = DK == 128 && DV == 128 ? 1 : DV == 128 ? 2 : 3;
+  static constexpr int kOffQ = 0;
+  static constexpr int kOffDO = 2 * kQBytes;
+  static constexpr int kOffK = kOffDO + 2 * kDOBytes;
+  static constexpr int kOffV = kOffK + kKStages * kKBytes;
+  static constexpr int kOffBar = kOffV + kVStages * kVBytes;
+  // barriers: k_full[KS], k_empty[KS], v_full[VS], v_empty[VS], q_full, then for each tile s_full,
+  // s_free, dp_full, ds_ready, done
+  static constexpr int kNumBars = 2 * (kKStages + kVStages) + 1 + 10;
+  static constexpr int kOffMisc = kOffBar + kNumBars * 8;
+  static constexpr int kSmemBytes = kOffMisc + 16 + 1024;
+  static constexpr uint32_t kTmemDQ = 256;  // X0 at 0, X1 at 128, dQ0 at 256, dQ1 at 256 + DK
+  static_assert(kTmemDQ + 2 * DK <= kTmemCols, "TMEM budget");
+  static_assert(kSmemBytes <= 232448, "shared memory budget");
+};
+
+template <int DK, int DV>
+__global__ void __launch_bounds__(Dq2Cfg<DK, DV>::kThreads, 1)
+attn_bwd_dq2_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
+                    const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmDO,
+                    const float* __restrict__ nL, const float* __restrict__ Dd,
+                    __nv_bfloat16* __restrict__ dQ, int Nq, int Nk, int Nq_pad, int n_qblocks,
+                    float c_log2, float scale, bool second, uint64_t wait_limit_ns) {
+  using C = Dq2Cfg<DK, DV>;
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
+                                             ~uintptr_t(1023));
+  const uint32_t sQ = smem_u32(smem + C::kOffQ);
+  const uint32_t sDO = smem_u32(smem + C::kOffDO);
+  const uint32_t sK = smem_u32(smem + C::kOffK);
+  const uint32_t sV = smem_u32(smem + C::kOffV);
+  const uint32_t bar0 = smem_u32(smem + C::kOffBar);
+  auto k_full = [&](int i) { return bar0 + 8u * i; };
+  auto k_empty = [&](int i) { return bar0 + 8u * (C::kKStages + i); };
+  const uint32_t bar_v = bar0 + 16u * C::kKStages;
+  auto v_full = [&](int i) { return bar_v + 8u * i; };
+  auto v_empty = [&](int i) { return bar_v + 8u * (C::kVStages + i); };
+  const uint32_t q_full = bar_v + 16u * C::kVStages;
+  auto s_full = [&](int j) { return q_full + 8 + 40u * j; };
+  auto s_free = [&](int j) { return q_full + 16 + 40u * j; };
+  auto dp_full = [&](int j) { return q_full + 24 + 40u * j; };
+  auto ds_ready = [&](int j) { return q_full + 32 + 40u * j; };
+  auto done = [&](int j) { return q_full + 40 + 40u * j; };
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + C::kOffMisc);
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + C::kOffMisc + 4);
+
+  const int warp = threadIdx.x >> 5;
+  const int lane = threadIdx.x & 31;
+  const int bh = blockIdx.x / n_qblocks;
+  const int q0 = (blockIdx.x % n_qblocks) * (2 * kBlk);
+  const int n_kb = (Nk + kBlk - 1) / kBlk;
+  const WaitCtl wc{abort_flag, wait_limit_ns, 0u, &g_moa_bwd_status};
+
+  if (threadIdx.x == 0) {
+    for (int i = 0; i < C::kKStages; ++i) {
+      mbar_init(k_full(i), 1);
+      mbar_init(k_empty(i), 2);  // one commit from each tile's issuer
+    }
+    for (int i = 0; i < C::kVStages; ++i) {
+      mbar_init(v_full(i), 1);
+      mbar_init(v_empty(i), 2);
+    }
+    mbar_init(q_full, 1);
+    for (int j = 0; j < 2; ++j) {
+      mbar_init(s_full(j), 1);
+      mbar_init(s_free(j), 128);
+      mbar_init(dp_full(j), 1);
+      mbar_init(ds_ready(j), 128);
+      mbar_init(done(j), 1);
+    }
+    *abort_flag = 0;
+    fence_barrier_init();
+  }
+  if (warp == C::kMmaWarp0) {
+    tmem_alloc(smem_u32(tmem_slot), kTmemCols);
+    tmem_relinquish();
+  }
+  tc_fence_before_sync();
+  __syncthreads();
+  tc_fence_after_sync();
+  const uint32_t tmem = *tmem_slot;
+  tile_kernel_begin(second);
+
+  if (warp >= 8) {
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(C::kRegsCtrl));
+    if (warp == C::kLoadWarp) {
+      // -------------------------------------------------------------- TMA producer
+      if (lane == 0) {
+        tma_prefetch_desc(&tmQ);
+        tma_prefetch_desc(&tmK);
+        tma_prefetch_desc(&tmV);
+        tma_prefetch_desc(&tmDO);
+        mbar_arrive_expect_tx(q_full, 2 * (C::kQBytes + C::kDOBytes));
+        for (int j = 0; j < 2; ++j) {
+#pragma unroll
+          for (int p = 0; p < DK / 64; ++p)
+            tma_load_3d(sQ + j * C::kQBytes + p * kPanelBytes, &tmQ, q_full, p * 64, q0 + j * kBlk, bh);
+#pragma unroll
+          for (int p = 0; p < DV / 64; ++p)
+            tma_load_3d(sDO + j * C::kDOBytes + p * kPanelBytes, &tmDO, q_full, p * 64, q0 + j * kBlk,
+                        bh);
+        }
+        int ks = 0, vs = 0;
+        uint32_t kph = 0, vph = 0, k_issued = 0, k_phase = 0, v_issued = 0, v_phase = 0;
+        bool aborted = false;
+        for (int n = 0; n < n_kb; ++n) {
+          if (!wait_bounded(k_empty(ks), kph ^ 1u, wc)) {
+            aborted = true;
+            break;
+          }
+          k_issued |= 1u << ks;
+          k_phase = (k_phase & ~(1u << ks)) | (kph << ks);
+          mbar_arrive_expect_tx(k_full(ks), C::kKBytes);
+#pragma unroll
+          for (int p = 0; p < DK / 64; ++p)
+            tma_load_3d(sK + ks * C::kKBytes + p * kPanelBytes, &tmK, k_full(ks), p * 64, n * kBlk, bh);
+          if (++ks == C::kKStages) {
+            ks = 0;
+            kph ^= 1u;
+          }
+          if (!wait_bounded(v_empty(vs), vph ^ 1u, wc)) {
+            aborted = true;
+            break;
+          }
+          v_issued |= 1u << vs;
+          v_phase = (v_phase & ~(1u << vs)) | (vph << vs);
+          mbar_arrive_expect_tx(v_full(vs), C::kVBytes);
+#pragma unroll
+          for (int p = 0; p < DV / 64; ++p)
+            tma_load_3d(sV + vs * C::kVBytes + p * kPanelBytes, &tmV, v_full(vs), p * 64, n * kBlk, bh);
+          if (++vs == C::kVStages) {
+            vs = 0;
+            vph ^= 1u;
+          }
+        }
+        if (aborted || *abort_flag) {
+          // Let every copy already issued land before the CTA can exit.
+          wait_quiesce(q_full, 0, wait_limit_ns, &g_moa_bwd_status);
+          for (int i = 0; i < C::kKStages; ++i)
+            if (k_issued & (1u << i))
+              wait_quiesce(k_full(i), (k_phase >> i) & 1u, wait_limit_ns, &g_moa_bwd_status);
+          for (int i = 0; i < C::kVStages; ++i)
+            if (v_issued & (1u << i))
+              wait_quiesce(v_full(i), (v_phase >> i) & 1u, wait_limit_ns, &g_moa_bwd_status);
+        }
+      }
+    } else if (warp == C::kMmaWarp0 || warp == C::kMmaWarp1) {
+      // -------------------------------------------------------------- MMA issuers
+      if (lane == 0) {
+        const int j = warp == C::kMmaWarp0 ? 0 : 1;
+        constexpr uint32_t kIdescS = make_idesc(kBlk, kBlk, false);
+        constexpr uint32_t kIdescDQ = make_idesc(kBlk, DK, true);
+        const uint32_t tX = tmem + 128u * j, tDQ = tmem + C::kTmemDQ + uint32_t(DK) * j;
+        const uint32_t sQj = sQ + j * C::kQBytes, sDOj = sDO + j * C::kDOBytes;
+        int ks = 0, vs = 0;
+        uint32_t kph = 0, vph = 0;
+        bool ok = wait_bounded(q_full, 0, wc);
+        for (int n = 0; ok && n < n_kb; ++n) {
+          const uint32_t par = uint32_t(n) & 1u;
+          // S = Q K^T (M = 128 queries, N = 128 keys, K-major operands); X holds dS(n-1), which
+          // dQ(n-1), issued before, has read by then (products of one CTA run in issue order).
+          ok = wait_bounded(k_full(ks), kph, wc);
+          if (!ok) break;
+          tc_fence_after_sync();
+          const uint32_t kt = sK + ks * C::kKBytes;
+#pragma unroll
+          for (int kk = 0; kk < DK / 16; ++kk) {
+            const uint32_t off = (kk >> 2) * kPanelBytes + (kk & 3) * 32;
+            mma_f16_ss(tX, make_sdesc_sw128(sQj + off, 16, 1024), make_sdesc_sw128(kt + off, 16, 1024),
+                       kIdescS, kk > 0 ? 1u : 0u);
+          }
+          mma_commit(s_full(j));
+          // dP = dO V^T over S, once the tile's threads hold S in registers
+          ok = wait_bounded(v_full(vs), vph, wc) && wait_bounded(s_free(j), par, wc);
+          if (!ok) break;
+          tc_fence_after_sync();
+          const uint32_t vt = sV + vs * C::kVBytes;
+#pragma unroll
+          for (int kk = 0; kk < DV / 16; ++kk) {
+            const uint32_t off = (kk >> 2) * kPanelBytes + (kk & 3) * 32;
+            mma_f16_ss(tX, make_sdesc_sw128(sDOj + off, 16, 1024), make_sdesc_sw128(vt + off, 16, 1024),
+                       kIdescS, kk > 0 ? 1u : 0u);
+          }
+          mma_commit(dp_full(j));
+          mma_commit(v_empty(vs));
+          if (++vs == C::kVStages) {
+            vs = 0;
+            vph ^= 1u;
+          }
+          // dQ += dS K (scale applied in the epilogue): A = dS (bf16 pairs, 8 columns per 16 keys),
+          // B = K tile MN-major.
+          ok = wait_bounded(ds_ready(j), par, wc);
+          if (!ok) break;
+          tc_fence_after_sync();
+#pragma unroll
+          for (int kk = 0; kk < kBlk / 16; ++kk)
+            mma_f16_ts(tDQ, tX + kk * 8, make_sdesc_sw128(kt + kk * 2048, kPanelBytes, 1024), kIdescDQ,
+                       (kk > 0 || n > 0) ? 1u : 0u);
+          mma_commit(k_empty(ks));
+          if (++ks == C::kKStages) {
+            ks = 0;
+            kph ^= 1u;
+          }
+        }
+        mma_commit(done(j));  // TMEM quiescent before it is freed, also on the abort path
+      }
+    }
+  } else {
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(C::kRegsCompute));
+    // ---------------------------------------------------------------- compute warpgroups
+    const int j = warp >> 2;
+    const int lane_base = (warp & 3) * 32;
+    const int row = q0 + j * kBlk + lane_base + lane;  // query row of this thread
+    const uint32_t lanes = uint32_t(lane_base) << 16;
+    const uint32_t tX = tmem + lanes + 128u * j;
+    // padded rows (past the array's Nq_pad as well) weigh nothing
+    const bool in = row < Nq_pad;
+    const size_t vrow = size_t(bh) * Nq_pad + size_t(in ? row : 0);
+    const float nl = in ? __ldcg(nL + vrow) : -INFINITY, dd = in ? __ldcg(Dd + vrow) : 0.f;
+    const uint64_t cc = pack_f32x2(c_log2, c_log2);
+    const uint64_t nn = pack_f32x2(nl, nl);
+    bool ok = true;
+    for (int n = 0; n < n_kb; ++n) {
+      const uint32_t par = uint32_t(n) & 1u;
+      ok = wait_bounded(s_full(j), par, wc);
+      if (!ok) break;
+      tc_fence_after_sync();
+      uint32_t sr[128];
+      tmem_load_row128(tX, sr);
+      tc_fence_before_sync();
+      mbar_arrive(s_free(j));  // S is in registers: dP may overwrite it
+      float* p = reinterpret_cast<float*>(sr);
+#pragma unroll
+      for (int k = 0; k < kBlk; k += 2) {
+        ffma2(p[k], p[k + 1], p[k], p[k + 1], cc, nn);
+        p[k] = ex2_approx(p[k]);
+        p[k + 1] = ex2_approx(p[k + 1]);
+      }
+      ok = wait_bounded(dp_full(j), par, wc);
+      if (!ok) break;
+      tc_fence_after_sync();
+      // dS = P (dP - D), 16 columns at a time, the next 16 on their way meanwhile; the 16 packed
+      // columns of chunks 2c and 2c + 1 lie at or below the columns of dP already read
+      uint32_t ra[16], rb[16], pk[16];
+      auto ds16 = [&](int c, const uint32_t* r, uint32_t* out) {
+#pragma unroll
+        for (int k = 0; k < 16; k += 2)
+          out[k >> 1] = pack_bf16x2(p[16 * c + k] * (__uint_as_float(r[k]) - dd),
+                                    p[16 * c + k + 1] * (__uint_as_float(r[k + 1]) - dd));
+      };
+      tmem_ld_32x32b_x16(tX, ra);
+#pragma unroll
+      for (int c = 0; c < 8; c += 2) {
+        tmem_wait_ld();
+        reg_anchor_x16(ra);
+        tmem_ld_32x32b_x16(tX + 16 * (c + 1), rb);
+        ds16(c, ra, pk);
+        tmem_wait_ld();
+        reg_anchor_x16(rb);
+        if (c + 2 < 8) tmem_ld_32x32b_x16(tX + 16 * (c + 2), ra);
+        ds16(c + 1, rb, pk + 8);
+        tmem_st_32x32b_x16(tX + 8 * c, pk);
+      }
+      tmem_wait_st();
+      tc_fence_before_sync();
+      mbar_arrive(ds_ready(j));
+    }
+    // Epilogue: scale * dQ -> bf16
+    if (ok && wait_bounded(done(j), 0, wc)) {
+      tc_fence_after_sync();
+      const bool valid = row < Nq;
+      __nv_bfloat16* dst = dQ + (size_t(bh) * Nq + size_t(valid ? row : 0)) * DK;
+      store_row_bf16<DK>(tmem + lanes + C::kTmemDQ + uint32_t(DK) * j, scale, dst, valid);
+    }
+  }
+
+  if (warp == C::kMmaWarp0) {
+    wait_quiesce(done(0), 0, wait_limit_ns, &g_moa_bwd_status);
+    wait_quiesce(done(1), 0, wait_limit_ns, &g_moa_bwd_status);
+  }
+  tc_fence_before_sync();
+  __syncthreads();
+  if (warp == C::kMmaWarp0) {
+    tc_fence_after_sync();
+    tmem_dealloc(tmem, kTmemCols);
+  }
+  tile_kernel_end(second);
 }
 
 
@@ -1210,20 +1537,31 @@ attn_bwd_dq_convert_kernel(const float* __restrict__ dq_acc, __nv_bfloat16* __re
 // ------------------------------------------------------------------------------------------
 int64_t padded_rows(int64_t Nq) { return (Nq + kBlk - 1) / kBlk * kBlk; }
 
+// Two query tiles per CTA where the estimated time is less: all CTAs' key blocks spread over the SMs
+// plus a third of the longest CTA, and at least that CTA.  In clocks per (query, key) block pair, from
+// launches that fill the GPU: dK/dV 3500, one-tile dQ 3250, two-tile dQ 4850 for two query blocks (d_k +
+// d_v > 128; 5300 for d = 64, whose products are shorter and whose exponentials are not).  The bits of
+// dQ are the same either way.
+// Measured, one -> two tiles on a GB300: 2x16x4096x4096 d=128 788 -> 706 us, 8x8x1024x4096 d_k=128
+// d_v=64 372 -> 358, 1x16x1000x3000 d=128 90 -> 81, 4x16x2048x2048 d=64 331 -> 314; the other way round 1x4x2048x2048 d=128 39 -> 49,
+// 3x5x500x1500 d=64 22 -> 30 (too few CTAs to fill the SMs).
+template <int DK, int DV>
+bool dq_two_tiles(int64_t BH, int64_t n_qb, int64_t n_kb, int sms) {
+  constexpr double kKv = 3500, kOne = 3250, kTwo = DK + DV > 128 ? 4850 : 5300;
+  auto time = [&](double blocks, double cost) {
+    const double work = double(BH) * double(n_kb) * (double(n_qb) * kKv + blocks * cost);
+    const double kv = double(n_qb) * kKv, dq = double(n_kb) * cost, chain = kv > dq ? kv : dq;
+    const double t = work / sms + 0.35 * chain;
+    return t > chain ? t : chain;
+  };
+  return time(double((n_qb + 1) / 2), kTwo) < time(double(n_qb), kOne);
+}
+
 template <int DK, int DV>
 int launch_bwd(const BwdArgs& a, const CUtensorMap& mq, const CUtensorMap& mk,
                const CUtensorMap& mv, const CUtensorMap& mdo, char* msg, size_t msglen) {
   using A = DkDvCfg<DK, DV>;
   using B = DqCfg<DK, DV>;
-  cudaError_t attr_err =
-      ensure_smem_limit(reinterpret_cast<const void*>(attn_bwd_dkdv_kernel<DK, DV>), A::kSmemBytes);
-  if (attr_err == cudaSuccess)
-    attr_err =
-        ensure_smem_limit(reinterpret_cast<const void*>(attn_bwd_dq_kernel<DK, DV>), B::kSmemBytes);
-  if (attr_err != cudaSuccess) {
-    snprintf(msg, msglen, "cudaFuncSetAttribute (bf16 backward): %s", cudaGetErrorString(attr_err));
-    return 5;
-  }
   const int64_t BH = a.B * a.H;
   const int64_t nq_pad = padded_rows(a.Nq);
   const int64_t n_kb = (a.Nk + kBlk - 1) / kBlk, n_qb = nq_pad / kBlk;
@@ -1231,6 +1569,31 @@ int launch_bwd(const BwdArgs& a, const CUtensorMap& mq, const CUtensorMap& mk,
       nq_pad > 0x7fffffffLL) {
     snprintf(msg, msglen, "bf16 backward: grid too large");
     return 3;
+  }
+  using D = Dq2Cfg<DK, DV>;
+  const int64_t n_q2 = (n_qb + 1) / 2;
+  int sms = 0;
+  cudaError_t pe = device_sm_count(&sms);
+  const bool two_tiles = pe == cudaSuccess && dq_two_tiles<DK, DV>(BH, n_qb, n_kb, sms);
+  if (two_tiles) {
+    // The register split moves registers inside the CTA's launch allocation: refuse a build whose
+    // allocation is short of the split's sum.
+    static std::atomic<int> regs = {-1};
+    if (regs.load(std::memory_order_relaxed) < 0) {
+      cudaFuncAttributes fa;
+      pe = cudaFuncGetAttributes(&fa, reinterpret_cast<const void*>(attn_bwd_dq2_kernel<DK, DV>));
+      if (pe == cudaSuccess) regs.store(fa.numRegs, std::memory_order_relaxed);
+    }
+    const int r = regs.load(std::memory_order_relaxed);
+    if (pe == cudaSuccess && r * D::kThreads < 256 * D::kRegsCompute + 128 * D::kRegsCtrl) {
+      snprintf(msg, msglen, "bf16 backward compiled to %d registers per thread, short of the register "
+               "split", r);
+      return 5;
+    }
+  }
+  if (pe != cudaSuccess) {
+    snprintf(msg, msglen, "bf16 backward set-up: %s", cudaGetErrorString(pe));
+    return 5;
   }
   float* nL = static_cast<float*>(a.ws);
   float* Dd = nL + BH * nq_pad;
@@ -1242,19 +1605,39 @@ int launch_bwd(const BwdArgs& a, const CUtensorMap& mq, const CUtensorMap& mk,
       dim3(256), 0, a.stream, static_cast<const __nv_bfloat16*>(a.O),
       static_cast<const __nv_bfloat16*>(a.dO), a.lse, nL, Dd, int(a.Nq), int(nq_pad), rows_pad,
       static_cast<float*>(nullptr));
+  auto launch_dkdv = [&](bool second) {
+    cudaError_t r = ensure_smem_limit(reinterpret_cast<const void*>(attn_bwd_dkdv_kernel<DK, DV>),
+                                      A::kSmemBytes);
+    if (r == cudaSuccess)
+      r = launch_dependent(attn_bwd_dkdv_kernel<DK, DV>, dim3(unsigned(BH * n_kb)), dim3(A::kThreads),
+                           A::kSmemBytes, a.stream, mq, mk, mv, mdo, static_cast<const float*>(nL),
+                           static_cast<const float*>(Dd), static_cast<__nv_bfloat16*>(a.dK),
+                           static_cast<__nv_bfloat16*>(a.dV), int(a.Nk), int(nq_pad), int(n_kb),
+                           c_log2, a.scale, second, wait_limit_ns());
+    return r;
+  };
+  auto launch_dq = [&](auto kern, int64_t blocks, int threads, int smem, bool second) {
+    cudaError_t r = ensure_smem_limit(reinterpret_cast<const void*>(kern), smem);
+    if (r == cudaSuccess)
+      r = launch_dependent(kern, dim3(unsigned(BH * blocks)), dim3(threads), smem, a.stream, mq, mk,
+                           mv, mdo, static_cast<const float*>(nL), static_cast<const float*>(Dd),
+                           static_cast<__nv_bfloat16*>(a.dQ), int(a.Nq), int(a.Nk), int(nq_pad),
+                           int(blocks), c_log2, a.scale, second, wait_limit_ns());
+    return r;
+  };
   if (e == cudaSuccess) {
-    e = launch_dependent(attn_bwd_dkdv_kernel<DK, DV>, dim3(unsigned(BH * n_kb)), dim3(A::kThreads),
-                         A::kSmemBytes, a.stream, mq, mk, mv, mdo, static_cast<const float*>(nL),
-                         static_cast<const float*>(Dd),
-                         static_cast<__nv_bfloat16*>(a.dK), static_cast<__nv_bfloat16*>(a.dV),
-                         int(a.Nk), int(nq_pad), int(n_kb), c_log2, a.scale, wait_limit_ns());
-  }
-  if (e == cudaSuccess) {
-    e = launch_dependent(attn_bwd_dq_kernel<DK, DV>, dim3(unsigned(BH * n_qb)), dim3(B::kThreads),
-                         B::kSmemBytes, a.stream, mq, mk, mv, mdo, static_cast<const float*>(nL),
-                         static_cast<const float*>(Dd),
-                         static_cast<__nv_bfloat16*>(a.dQ), int(a.Nq), int(a.Nk), int(nq_pad),
-                         int(n_qb), c_log2, a.scale, wait_limit_ns());
+    if (two_tiles) {
+      // its CTAs run longest: first
+      e = launch_dq(attn_bwd_dq2_kernel<DK, DV>, n_q2, D::kThreads, D::kSmemBytes, false);
+      if (e == cudaSuccess) e = launch_dkdv(true);
+    } else if (n_qb >= n_kb) {  // the longer CTAs first
+      e = launch_dkdv(false);
+      if (e == cudaSuccess)
+        e = launch_dq(attn_bwd_dq_kernel<DK, DV>, n_qb, B::kThreads, B::kSmemBytes, true);
+    } else {
+      e = launch_dq(attn_bwd_dq_kernel<DK, DV>, n_qb, B::kThreads, B::kSmemBytes, false);
+      if (e == cudaSuccess) e = launch_dkdv(true);
+    }
   }
   if (e != cudaSuccess) {
     snprintf(msg, msglen, "bf16 backward launch: %s", cudaGetErrorString(e));
