@@ -1537,24 +1537,41 @@ attn_bwd_dq_convert_kernel(const float* __restrict__ dq_acc, __nv_bfloat16* __re
 // ------------------------------------------------------------------------------------------
 int64_t padded_rows(int64_t Nq) { return (Nq + kBlk - 1) / kBlk * kBlk; }
 
-// Two query tiles per CTA where the estimated time is less: all CTAs' key blocks spread over the SMs
-// plus a third of the longest CTA, and at least that CTA.  In clocks per (query, key) block pair, from
-// launches that fill the GPU: dK/dV 3500, one-tile dQ 3250, two-tile dQ 4850 for two query blocks (d_k +
-// d_v > 128; 5300 for d = 64, whose products are shorter and whose exponentials are not).  The bits of
-// dQ are the same either way.
+// Estimated clocks of the two tile kernels of the three-kernel path: all CTAs' blocks spread over the
+// SMs plus a quarter of the longest CTA, and at least that CTA.  Per (query, key) block pair, from
+// launches that fill the GPU: dK/dV 3500, one-tile dQ 3250, two-tile dQ 4850 for two query blocks at
+// d_k + d_v > 128; 2750, 2650 and 4950 at d = 64; and 6000 to start and end a CTA.
+template <int DK, int DV>
+double three_kernel_clocks(int64_t BH, int64_t n_qb, int64_t n_kb, int sms, bool two_tiles) {
+  constexpr bool kBig = DK + DV > 128;
+  constexpr double kKv = kBig ? 3500 : 2750, kOne = kBig ? 3250 : 2650, kTwo = kBig ? 4850 : 4950;
+  constexpr double kCta = 6000;
+  const double kv = double(n_qb) * kKv + kCta;
+  const double dq = double(n_kb) * (two_tiles ? kTwo : kOne) + kCta;
+  const double ctas_q = double(two_tiles ? (n_qb + 1) / 2 : n_qb);
+  const double chain = kv > dq ? kv : dq;
+  const double t = double(BH) * (double(n_kb) * kv + ctas_q * dq) / sms + 0.25 * chain;
+  return t > chain ? t : chain;
+}
+// Two query tiles per dQ CTA where that takes less.
 // Measured, one -> two tiles on a GB300: 2x16x4096x4096 d=128 788 -> 706 us, 8x8x1024x4096 d_k=128
-// d_v=64 372 -> 358, 1x16x1000x3000 d=128 90 -> 81, 4x16x2048x2048 d=64 331 -> 314; the other way round 1x4x2048x2048 d=128 39 -> 49,
-// 3x5x500x1500 d=64 22 -> 30 (too few CTAs to fill the SMs).
+// d_v=64 372 -> 358, 1x16x1000x3000 d=128 90 -> 81, 4x16x2048x2048 d=64 331 -> 314; the other way round
+// 1x4x2048x2048 d=128 39 -> 49, 3x5x500x1500 d=64 22 -> 30 (too few CTAs to fill the SMs).
 template <int DK, int DV>
 bool dq_two_tiles(int64_t BH, int64_t n_qb, int64_t n_kb, int sms) {
-  constexpr double kKv = 3500, kOne = 3250, kTwo = DK + DV > 128 ? 4850 : 5300;
-  auto time = [&](double blocks, double cost) {
-    const double work = double(BH) * double(n_kb) * (double(n_qb) * kKv + blocks * cost);
-    const double kv = double(n_qb) * kKv, dq = double(n_kb) * cost, chain = kv > dq ? kv : dq;
-    const double t = work / sms + 0.35 * chain;
-    return t > chain ? t : chain;
-  };
-  return time(double((n_qb + 1) / 2), kTwo) < time(double(n_qb), kOne);
+  return three_kernel_clocks<DK, DV>(BH, n_qb, n_kb, sms, true) <
+         three_kernel_clocks<DK, DV>(BH, n_qb, n_kb, sms, false);
+}
+// Whether the three kernels take less than the fused one (d = 64): rounds of fused CTAs at 3700 clocks
+// per block pair and 7000 per CTA, its accumulator zeroed and converted; both with their launches.
+// Measured, fused / three kernels on a GB300 (us): 1x1x92x92 9.3 / 6.4, 6x8x661x84 22.1 / 15.4,
+// 3x5x500x1500 27.9 / 22.1, 1x1x8000x8000 122 / 95; 1x16x1024x1024 25.6 / 28.5, 4x16x2048x2048 255 / 314.
+bool fused_takes_three(int64_t BH, int64_t n_qb, int64_t n_kb, int sms) {
+  const double one = three_kernel_clocks<64, 64>(BH, n_qb, n_kb, sms, false);
+  const double two = three_kernel_clocks<64, 64>(BH, n_qb, n_kb, sms, true);
+  const double rounds = double((BH * n_kb + sms - 1) / sms);
+  const double fused = rounds * (double(n_qb) * 3700 + 7000) + 0.16 * double(BH * n_qb * kBlk) + 5000;
+  return (one < two ? one : two) + 5200 < 0.97 * (fused + 8300);
 }
 
 template <int DK, int DV>
@@ -1714,6 +1731,14 @@ int launch_attn_bwd_bf16_fused(const BwdArgs& a, char* msg, size_t msglen) {
   if (!encode_bf16_map(&mk, a.K, BH, a.Nk, a.dk, msg, msglen)) return 5;
   if (!encode_bf16_map(&mv, a.V, BH, a.Nk, a.dv, msg, msglen)) return 5;
   if (!encode_bf16_map(&mdo, a.dO, BH, a.Nq, a.dv, msg, msglen)) return 5;
+  int sms = 0;
+  const cudaError_t e = device_sm_count(&sms);
+  if (e != cudaSuccess) {
+    snprintf(msg, msglen, "fused backward set-up: %s", cudaGetErrorString(e));
+    return 5;
+  }
+  const int64_t n_qb = (a.Nq + kBlk - 1) / kBlk, n_kb = (a.Nk + kBlk - 1) / kBlk;
+  if (fused_takes_three(BH, n_qb, n_kb, sms)) return launch_bwd<64, 64>(a, mq, mk, mv, mdo, msg, msglen);
   return launch_bwd_fused<64, 64>(a, mq, mk, mv, mdo, msg, msglen);
 }
 
