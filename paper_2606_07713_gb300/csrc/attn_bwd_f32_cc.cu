@@ -17,8 +17,8 @@
 // blocks of S and dP and R x 4C blocks of the gradients in registers; tiles, lane map and the
 // split over key groups are those of the fp32 forward kernel.
 // Measured on a GB300 (2070 MHz; before: one scalar shared load per operand and FMA, 32-row tiles):
-// 1x8x1024x1024 d=64 1016 -> 228 us (23.6 TFLOP/s of the five algorithmic products), 1x16x512x512
-// d=128 1550 -> 219 us.
+// 1x8x1024x1024 d=64 1016 -> 221 us (24.3 TFLOP/s of the five algorithmic products), d=128 1646 ->
+// 401 us; two iterations of the product loops together are worth 4 % of it.
 #include <cuda_runtime.h>
 #include <math.h>
 #include <cstdio>
@@ -182,7 +182,7 @@ __device__ __forceinline__ void bwd_rows(const float* __restrict__ A1, const flo
     for (int r = 0; r < R; ++r)
 #pragma unroll
       for (int j = 0; j < 8; ++j) x[r][j] = 0.f;
-#pragma unroll 1
+#pragma unroll 2
     for (int f = 0; f < d; f += 4) {
       float4 kk[8];
 #pragma unroll
@@ -211,7 +211,7 @@ __device__ __forceinline__ void bwd_rows(const float* __restrict__ A1, const flo
 #pragma unroll
         for (int j = 0; j < 4; ++j) myP[4 * r * kLdp + cg + 8 * j] = x[r][4 * half + j];
       __syncwarp();
-#pragma unroll 1
+#pragma unroll 2
       for (int k = 0; k < kHalf; k += 4) {
         float4 vv[4][C];
 #pragma unroll

@@ -74,6 +74,8 @@ attn_fwd_f32_cc_kernel(const float* __restrict__ Q, const float* __restrict__ K,
                        float scale) {
   using T = F32Tile<VC, R, WR, KW>;
   constexpr int kThreads = T::kThreads, kBM = T::kBM, kStep = T::kStep, kLdv = T::kLdv;
+  // two iterations of the product loops together: 2 to 5 % where registers are left (R <= 4)
+  constexpr int kUnroll = R == 8 ? 1 : 2;
   extern __shared__ __align__(16) float smem[];
   const int ldk = odd_stride(dk);
   float* sQ = smem;                // [kBM][ldk]
@@ -142,7 +144,7 @@ attn_fwd_f32_cc_kernel(const float* __restrict__ Q, const float* __restrict__ K,
 #pragma unroll
       for (int j = 0; j < 8; ++j) s[r][j] = 0.f;
     const int f_end = live ? dk : 0;
-#pragma unroll 1
+#pragma unroll kUnroll
     for (int f = 0; f < f_end; f += 4) {
       float4 kk[8];
 #pragma unroll
@@ -200,7 +202,7 @@ attn_fwd_f32_cc_kernel(const float* __restrict__ Q, const float* __restrict__ K,
 #pragma unroll
           for (int j = 0; j < 4; ++j) myP[4 * r * kLdp + cg + 8 * j] = s[r][4 * half + j];
         __syncwarp();
-#pragma unroll 1
+#pragma unroll kUnroll
         for (int k = 0; k < kHalf; k += 4) {
           float4 vv[4][VC];
 #pragma unroll
