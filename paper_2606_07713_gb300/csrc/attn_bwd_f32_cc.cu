@@ -263,6 +263,7 @@ __device__ __forceinline__ void bwd_rows(const float* __restrict__ A1, const flo
     if (left > kStep) request_step(k0 + kStep);
   }
 
+  launch_dependents();  // not before: see the bf16 forward on CTAs that share an SM
   if constexpr (KW > 1) {
     // Sum over the groups, in their order: groups g > 0 leave theirs where the tiles were
     // (thread-private slots, lane-contiguous).
@@ -323,7 +324,6 @@ attn_bwd_f32_kernel(const float* __restrict__ Q, const float* __restrict__ K,
                     float scale) {
   extern __shared__ __align__(16) float smem[];
   constexpr int kBM = BwdTile<C, R, WR, KW>::kBM;
-  launch_dependents();
   grid_dependency_wait();
   if (blockIdx.x < n_dkdv) {
     const long long bh = blockIdx.x / n_ktiles;

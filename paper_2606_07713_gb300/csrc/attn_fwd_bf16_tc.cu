@@ -253,7 +253,11 @@ attn_fwd_bf16_tc_kernel(const __grid_constant__ CUtensorMap tmQ,
   __syncthreads();
   tc_fence_after_sync();
   const uint32_t tmem = *tmem_slot;
-  launch_dependents();      // what follows on the stream may take SMs as they come free
+  // What follows on the stream may take SMs as they come free.  Where two CTAs share an SM this comes
+  // only after the key loop: CTAs of the next call that move in beside this one's, on whichever SMs
+  // have room, would run two to an SM with others idle (1x102x10x43657 d=64, call after call: 325 us,
+  // 402 with it here).
+  if constexpr (C::kMinBlocks == 1) launch_dependents();
   grid_dependency_wait();   // what came before has ended: its results are visible
 
   if (warp >= 4 * QT) {
@@ -525,6 +529,8 @@ attn_fwd_bf16_tc_kernel(const __grid_constant__ CUtensorMap tmQ,
       tc_fence_before_sync();
       mbar_arrive(p_ready(j));
     }
+    // (Past 64 key blocks, some 60 us, the launch saved is not worth the unevenness that is left.)
+    if (C::kMinBlocks > 1 && n_kt <= 64) launch_dependents();
     // Natural-log LSE of the scaled scores, final once the loop is done: m and l are in log2
     // units of c_log2 * s, and l is relative to m whether or not the last maximum update was
     // taken (lazy rescale).

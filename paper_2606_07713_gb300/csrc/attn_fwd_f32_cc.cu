@@ -109,7 +109,6 @@ attn_fwd_f32_cc_kernel(const float* __restrict__ Q, const float* __restrict__ K,
         *reinterpret_cast<float4*>(dst + (r - row0) * ld) = make_float4(0.f, 0.f, 0.f, 0.f);
     }
   };
-  launch_dependents();
   grid_dependency_wait();
   request(sQ, ldk, Qh, dk, q0, kBM, Nq);
   request(sK, ldk, Kh, dk, 0, kStep, Nk);
@@ -232,6 +231,7 @@ attn_fwd_f32_cc_kernel(const float* __restrict__ Q, const float* __restrict__ K,
     cp_async_commit();
   }
 
+  launch_dependents();  // not before: see the bf16 kernel on CTAs that share an SM
   if constexpr (KW > 1) {
     // Merge of the key groups: O = sum_g e^(m_g - M) O_g, l = sum_g e^(m_g - M) l_g, M = max m_g.
     // Groups g > 0 leave their state where the tiles were (thread-private slots, lane-contiguous).

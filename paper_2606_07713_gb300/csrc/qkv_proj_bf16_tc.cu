@@ -384,7 +384,6 @@ qkv_proj_small_kernel(const __grid_constant__ CUtensorMap tmX,
   __syncthreads();
   tc_fence_after_sync();
   const uint32_t tmem = *tmem_slot;
-  launch_dependents();     // what follows on the stream may take SMs as they come free
   grid_dependency_wait();  // what came before has ended: its results are visible
 
   if (warp == 0) {
@@ -443,6 +442,7 @@ qkv_proj_small_kernel(const __grid_constant__ CUtensorMap tmX,
     __syncwarp();
     wait_quiesce(drain, 0, wait_limit_ns, &g_moa_proj_status);
   } else if (wait_bounded(drain, 0, wc)) {
+    launch_dependents();  // not before: see the bf16 forward on CTAs that share an SM
     // The products have read every stage: the ring's memory now takes the partial sums.
     tc_fence_after_sync();
     const int col = (warp & 3) * 32 + lane;
