@@ -32,6 +32,9 @@
 // rows): work item = (b*H + h, block of 128 query rows); warps 0-3 softmax + epilogue, warp 4 TMEM
 // allocation and tcgen05.mma, warp 5 TMA loads.  At d_k = d_v = 64 two CTAs share an SM (256 TMEM
 // columns and ~98 KB of shared memory each); otherwise one CTA with a 6-stage ring.
+// DUP (split key axis, at most 128 query rows, d_v = 64): the two-tile kernel with both tiles on the
+// same 128 rows, tile 0 on the even and tile 1 on the odd key blocks, each with its own half of the
+// ring (warp 11 loads tile 1's); the two states are merged through shared memory at the end.
 // K and V tiles of 128 keys stream through an NS-stage shared-memory ring, in the order the
 // products use them: K0 K1 V0 K2 V1 ...  TMEM columns: S0 S1 P0 P1 O0 O1 at d_v = 64; one S
 // buffer shared by the two tiles, S P0 P1 O0 O1, at d_v = 128 (the two O take 256 columns);
@@ -74,10 +77,14 @@ constexpr float kRescaleLog2 = 8.0f;  // lazy-rescale threshold: exponentials st
 // costs 4 % at d_v = 128 (1712 -> 1638 TFLOP/s on 2x32x8192^2), where the MMA issuers' waits are
 // on the critical path; the one-tile kernel ran at 709 instead of 740 with it.
 
-template <int DK, int DV, int QT = 2>
+template <int DK, int DV, int QT = 2, bool DUP = false>
 struct Cfg {
   static_assert(DK == 64 || DK == 128, "d_k must be 64 or 128");
   static_assert(QT == 1 || QT == 2, "one or two Q tiles per CTA");
+  // DUP: both tiles are the same 128 query rows, and take the even and the odd key blocks, each with
+  // a ring, a producer and an issuer of its own.
+  static_assert(!DUP || (QT == 2 && DV == 64), "two S buffers need d_v = 64");
+  static constexpr int kQLoads = DUP ? 1 : QT;  // Q tiles in shared memory
   // Warps: 4 softmax warps per Q tile, then the MMA warp of tile 0 (it also allocates and frees
   // TMEM), the TMA warp and, with two tiles, the MMA warp of tile 1.  One-tile CTAs of d = 64 run
   // two per SM (half the registers, TMEM and shared memory each).
@@ -115,14 +122,15 @@ struct Cfg {
   // the same; it moves 128 KB more per key block through shared memory.)  One tile: S0 P0 O0.
   static constexpr bool kSharedS = QT == 2 && DV == 128;
   static constexpr int kStages = QT == 1 ? (kMinBlocks == 2 ? 5 : 6)
+                                 : DUP ? (DK == 64 ? 12 : 6)  // half per ring
                                  : (DK == 64 && DV == 64) ? 8
                                  : kSharedS ? (DK == 128 ? 5 : 6) : 4;
   static constexpr int kOffQ = 0;
-  static constexpr int kOffKV = kOffQ + QT * kQTileBytes;
+  static constexpr int kOffKV = kOffQ + kQLoads * kQTileBytes;
   static constexpr int kOffBar = kOffKV + kStages * kStageBytes;
   // Each Q tile gets its own issuing thread (its chain of products never waits behind the
   // other tile's).
-  static constexpr int kIssuers = QT;
+  static constexpr int kIssuers = DUP ? 1 : QT;  // of one stage
   // Chunks of 32 exponentials computed before the wait for P's buffer (the rest after it), so
   // that the wait for the previous block's P V overlaps them (measured on 4x16x2048^2, d=64:
   // 0 -> 2 chunks 740 -> 812 TFLOP/s; 1x16x32768^2, d=128: 0 -> 3 chunks +2 %; with the
@@ -178,17 +186,20 @@ __device__ __forceinline__ void tmem_scale_row(uint32_t taddr, float alpha) {
 
 // SPLIT: this CTA covers one range of the key axis and writes fp32 partials for the merge kernel
 // (separate instantiation, so the unsplit kernel carries none of it).
-template <int DK, int DV, bool SPLIT, int QT>
-__global__ void __launch_bounds__(Cfg<DK, DV, QT>::kThreads, Cfg<DK, DV, QT>::kMinBlocks)
+template <int DK, int DV, bool SPLIT, int QT, bool DUP = false>
+__global__ void __launch_bounds__(Cfg<DK, DV, QT, DUP>::kThreads, Cfg<DK, DV, QT, DUP>::kMinBlocks)
 attn_fwd_bf16_tc_kernel(const __grid_constant__ CUtensorMap tmQ,
                         const __grid_constant__ CUtensorMap tmK,
                         const __grid_constant__ CUtensorMap tmV, __nv_bfloat16* __restrict__ O,
                         int Nq, int Nk, int n_qblocks, float c_log2, uint64_t wait_limit_ns,
                         int n_splits, int kv_per_split, float* __restrict__ ws_o,
                         float2* __restrict__ ws_ml, float* __restrict__ lse) {
-  using C = Cfg<DK, DV, QT>;
+  using C = Cfg<DK, DV, QT, DUP>;
   constexpr int kQTiles = QT;
+  constexpr int kStep = DUP ? 2 : 1;             // a tile takes every kStep-th key block
+  constexpr int kRing = C::kStages / kStep;      // stages of one ring
   constexpr int kMmaWarp0 = C::kMmaWarp0, kLoadWarp = C::kLoadWarp, kMmaWarp1 = C::kMmaWarp1;
+  constexpr int kLoadWarp1 = 11;  // DUP only
   constexpr int kTmemCols = C::kTmemCols;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
@@ -219,7 +230,7 @@ attn_fwd_bf16_tc_kernel(const __grid_constant__ CUtensorMap tmQ,
   const int split = SPLIT ? int(blockIdx.x % n_splits) : 0;
   const int item = SPLIT ? int(blockIdx.x / n_splits) : int(blockIdx.x);
   const int bh = item / n_qblocks;
-  const int q0 = (item % n_qblocks) * (kQTiles * kBM);
+  const int q0 = (item % n_qblocks) * (C::kQLoads * kBM);
   // This CTA's key blocks: [kb0, kb0 + n_kt) (all of them unless the key axis is split).
   const int kb0 = SPLIT ? split * kv_per_split : 0;
   const int n_kt = SPLIT ? min((Nk + kBN - 1) / kBN - kb0, kv_per_split) : (Nk + kBN - 1) / kBN;
@@ -264,25 +275,30 @@ attn_fwd_bf16_tc_kernel(const __grid_constant__ CUtensorMap tmQ,
     // Control warps (MMA issuers, TMA producer, and with two tiles an idle warp).
     if constexpr (C::kRegSplit)
       asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(C::kRegsCtrl));
-  if (warp == kLoadWarp) {
-    // ---------------------------------------------------------------- TMA producer
+  if (warp == kLoadWarp || (DUP && warp == kLoadWarp1)) {
+    // ---------------------------------------------------------------- TMA producer (DUP: one per tile)
     if (lane == 0) {
+      const int first = DUP && warp == kLoadWarp1 ? 1 : 0;  // first key block of this ring
+      const int ring0 = first * kRing;                      // its first stage
+      const int n_mine = (n_kt - first + kStep - 1) / kStep;
       tma_prefetch_desc(&tmQ);
       tma_prefetch_desc(&tmK);
       tma_prefetch_desc(&tmV);
-      mbar_arrive_expect_tx(q_full, kQTiles * C::kQTileBytes);
-      for (int j = 0; j < kQTiles; ++j)
+      if (first == 0) {
+        mbar_arrive_expect_tx(q_full, C::kQLoads * C::kQTileBytes);
+        for (int j = 0; j < C::kQLoads; ++j)
 #pragma unroll
-        for (int p = 0; p < DK / 64; ++p)
-          tma_load_3d(sQ + j * C::kQTileBytes + p * C::kPanelBytes, &tmQ, q_full, p * 64,
-                      q0 + j * kBM, bh);
-      int slot = 0;
+          for (int p = 0; p < DK / 64; ++p)
+            tma_load_3d(sQ + j * C::kQTileBytes + p * C::kPanelBytes, &tmQ, q_full, p * 64,
+                        q0 + j * kBM, bh);
+      }
+      int slot = ring0;
       uint32_t phase = 0;
       uint32_t issued = 0, issued_phase = 0;  // per slot: a load was issued / its phase bit
       bool aborted = false;
       // Ring order = the MMA issuers' consumption order: K0 K1 V0 K2 V1 ... (block n+1's scores
       // come before block n's P V).
-      for (int t = 0; t < 2 * n_kt; ++t) {
+      for (int t = 0; t < 2 * n_mine; ++t) {
         bool is_k;
         int n;
         if (t == 0) {
@@ -290,9 +306,10 @@ attn_fwd_bf16_tc_kernel(const __grid_constant__ CUtensorMap tmQ,
           n = 0;
         } else {
           const int u = t - 1, nn = u >> 1;
-          is_k = (u & 1) == 0 && nn + 1 < n_kt;
+          is_k = (u & 1) == 0 && nn + 1 < n_mine;
           n = is_k ? nn + 1 : nn;
         }
+        n = first + kStep * n;
         if (!wait_bounded(empty_bar(slot), phase ^ 1u, wc)) {
           aborted = true;
           break;
@@ -313,14 +330,14 @@ attn_fwd_bf16_tc_kernel(const __grid_constant__ CUtensorMap tmQ,
             tma_load_3d(dst + p * C::kPanelBytes, &tmV, full_bar(slot), p * 64, (kb0 + n) * kBN,
                         bh);
         }
-        if (++slot == C::kStages) {
-          slot = 0;
+        if (++slot == ring0 + kRing) {
+          slot = ring0;
           phase ^= 1u;
         }
       }
       if (aborted || *abort_flag) {
         // Let every copy already issued land before the CTA can exit.
-        wait_quiesce(q_full, 0, wait_limit_ns, &g_moa_bf16_status);
+        if (first == 0) wait_quiesce(q_full, 0, wait_limit_ns, &g_moa_bf16_status);
         for (int sl = 0; sl < C::kStages; ++sl)
           if (issued & (1u << sl))
             wait_quiesce(full_bar(sl), (issued_phase >> sl) & 1u, wait_limit_ns, &g_moa_bf16_status);
@@ -338,14 +355,16 @@ attn_fwd_bf16_tc_kernel(const __grid_constant__ CUtensorMap tmQ,
       const uint32_t tS = tmem + (j ? C::kTmemS1 : C::kTmemS0);
       const uint32_t tP = tmem + (j ? C::kTmemP1 : C::kTmemP0);
       const uint32_t tO = tmem + (j ? C::kTmemO1 : C::kTmemO0);
-      const uint32_t sQj = sQ + j * C::kQTileBytes;
+      const uint32_t sQj = DUP ? sQ : sQ + j * C::kQTileBytes;
+      const int ring0 = DUP ? j * kRing : 0;
+      const int n_mine = DUP ? (n_kt - j + 1) / 2 : n_kt;
       const uint32_t bar_s_full = s_full(j), bar_p_ready = p_ready(j), bar_s_free = s_free(j);
       const uint32_t bar_p_free = p_free(j);
-      int slot = 0;
+      int slot = ring0;
       uint32_t phase = 0;
       auto next = [&]() {
-        if (++slot == C::kStages) {
-          slot = 0;
+        if (++slot == ring0 + kRing) {
+          slot = ring0;
           phase ^= 1u;
         }
       };
@@ -368,12 +387,13 @@ attn_fwd_bf16_tc_kernel(const __grid_constant__ CUtensorMap tmQ,
           mma_f16_ts(tO, tP + kk * 8, make_sdesc_sw128(vb + kk * 2048, C::kPanelBytes, 1024),
                      kIdescPV, kk > 0 ? 1u : acc_first);
       };
-      bool ok = wait_bounded(q_full, 0, wc) && wait_bounded(full_bar(slot), phase, wc);
+      bool ok = (!DUP || n_mine > 0) && wait_bounded(q_full, 0, wc) &&
+                wait_bounded(full_bar(slot), phase, wc);
       // Tile 1's first scores wait until tile 0 holds its own in registers: required with one
       // S buffer for both tiles (d_v = 128); with an S buffer per tile and d_k = 128 it keeps
       // the tiles' reads of S from tensor memory from coinciding (measured +2 % on
       // 8x8x1024x4096, d_k = 128, d_v = 64; -2 % with d_k = 64, which therefore starts both).
-      if ((DK == 128 || C::kSharedS) && j == 1) ok = ok && wait_bounded(s_free(0), 0, wc);
+      if (!DUP && (DK == 128 || C::kSharedS) && j == 1) ok = ok && wait_bounded(s_free(0), 0, wc);
       if (ok) {
         tc_fence_after_sync();
         const int ks = slot;
@@ -385,9 +405,9 @@ attn_fwd_bf16_tc_kernel(const __grid_constant__ CUtensorMap tmQ,
       {
         // P_j has TMEM columns of its own: S_j(n+1) is issued as soon as the S buffer's last
         // reader has its scores in registers, and O_j += P_j(n) V(n) once P_j(n) is written.
-        for (int n = 0; ok && n < n_kt; ++n) {
+        for (int n = 0; ok && n < n_mine; ++n) {
           const uint32_t par = uint32_t(n) & 1u;
-          if (n + 1 < n_kt) {
+          if (n + 1 < n_mine) {
             const int ks = slot;
             // The S buffer may take block n+1's scores once its last reader has them in
             // registers: this tile's softmax (own S buffer), or with one S buffer shared by the
@@ -431,7 +451,8 @@ attn_fwd_bf16_tc_kernel(const __grid_constant__ CUtensorMap tmQ,
     float m = -INFINITY;  // running maximum of c_log2 * s (log2 units)
     float l = 0.f;        // running sum of exp2(c_log2 * s - m)
     bool ok = true;
-    for (int n = 0; n < n_kt; ++n) {
+    const int n_mine = DUP ? (n_kt - j + 1) / 2 : n_kt;
+    for (int n = 0; n < n_mine; ++n) {
       if (!wait_bounded(s_full(j), uint32_t(n) & 1u, wc)) {
         ok = false;
         break;
@@ -444,7 +465,8 @@ attn_fwd_bf16_tc_kernel(const __grid_constant__ CUtensorMap tmQ,
       mbar_arrive(s_free(j));
       float* s = reinterpret_cast<float*>(sr);
       // Keys of this tile that exist.
-      const int valid = SPLIT ? min(kBN, *keys_from - n * kBN) : min(kBN, Nk - (kb0 + n) * kBN);
+      const int blk = DUP ? 2 * n + j : n;
+      const int valid = SPLIT ? min(kBN, *keys_from - blk * kBN) : min(kBN, Nk - (kb0 + blk) * kBN);
       // Step I: maximum of the scaled scores of this tile (max of s if c >= 0, else of -s).
       float tmax;
       if (valid == kBN) {
@@ -531,6 +553,76 @@ attn_fwd_bf16_tc_kernel(const __grid_constant__ CUtensorMap tmQ,
     }
     // (Past 64 key blocks, some 60 us, the launch saved is not worth the unevenness that is left.)
     if (C::kMinBlocks > 1 && n_kt <= 64) launch_dependents();
+    if constexpr (DUP) {
+      // Merge of the two tiles' key blocks (the identity of the split merge): tile 1 leaves its m, l
+      // and O in its ring, whose loads its products have all read; tile 0 takes them up.
+      float* mrg = reinterpret_cast<float*>(smem + C::kOffKV + kRing * C::kStageBytes);
+      static_assert((DV + 2) * kBM * 4 <= kRing * C::kStageBytes, "merge space");
+      const bool both = n_kt > 1;
+      if (j == 1 && both) {
+        ok = ok && wait_bounded(o_done(1), 0, wc);
+        tc_fence_after_sync();
+        mrg[row] = m;
+        mrg[kBM + row] = l;
+#pragma unroll
+        for (int c = 0; c < DV; c += 32) {
+          uint32_t o[32];
+          tmem_ld_32x32b_x32(tO + c, o);
+          tmem_wait_ld();
+          reg_anchor_x32(o);
+#pragma unroll
+          for (int i = 0; i < 32; ++i) mrg[(2 + c + i) * kBM + row] = __uint_as_float(o[i]);
+        }
+      }
+      asm volatile("barrier.sync 1, 256;" ::: "memory");  // the eight softmax warps
+      float w0 = 1.f, w1 = 0.f;
+      if (j == 0 && both) {
+        const float mo = mrg[row], mm = fmaxf(m, mo);
+        w0 = ex2_approx(m - mm);
+        w1 = ex2_approx(mo - mm);
+        m = mm;
+        l = fmaf(mrg[kBM + row], w1, l * w0);
+      }
+      const int grow = q0 + row;
+      if (j == 0 && ok && wait_bounded(o_done(0), 0, wc)) {
+        tc_fence_after_sync();
+        const float inv_l = SPLIT ? 1.0f : 1.0f / l;
+        if (!SPLIT && lse != nullptr && grow < Nq)
+          lse[size_t(bh) * Nq + grow] = (m + lg2_approx(l)) * 0.69314718055994531f;
+        const size_t prow =
+            SPLIT ? (size_t(*split_s) * (gridDim.x / n_splits / n_qblocks) + bh) * Nq + grow : 0;
+        if (SPLIT && grow < Nq) ws_ml[prow] = make_float2(m, l);
+#pragma unroll
+        for (int c = 0; c < DV; c += 16) {
+          uint32_t o[16];
+          tmem_ld_32x32b_x16(tO + c, o);
+          tmem_wait_ld();
+          reg_anchor_x16(o);
+          float v[16];
+#pragma unroll
+          for (int i = 0; i < 16; ++i) {
+            v[i] = __uint_as_float(o[i]) * w0;
+            if (both) v[i] = fmaf(mrg[(2 + c + i) * kBM + row], w1, v[i]);
+          }
+          if (grow < Nq) {
+            if constexpr (SPLIT) {
+              float4* dst = reinterpret_cast<float4*>(ws_o + prow * DV + c);
+#pragma unroll
+              for (int i = 0; i < 4; ++i)
+                dst[i] = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
+            } else {
+              uint4* dst = reinterpret_cast<uint4*>(O + (size_t(bh) * Nq + grow) * DV + c);
+#pragma unroll
+              for (int i = 0; i < 2; ++i)
+                dst[i] = make_uint4(pack_bf16x2(v[8 * i] * inv_l, v[8 * i + 1] * inv_l),
+                                    pack_bf16x2(v[8 * i + 2] * inv_l, v[8 * i + 3] * inv_l),
+                                    pack_bf16x2(v[8 * i + 4] * inv_l, v[8 * i + 5] * inv_l),
+                                    pack_bf16x2(v[8 * i + 6] * inv_l, v[8 * i + 7] * inv_l));
+            }
+          }
+        }
+      }
+    } else {
     // Natural-log LSE of the scaled scores, final once the loop is done: m and l are in log2
     // units of c_log2 * s, and l is relative to m whether or not the last maximum update was
     // taken (lazy rescale).
@@ -581,6 +673,7 @@ attn_fwd_bf16_tc_kernel(const __grid_constant__ CUtensorMap tmQ,
           for (int i = 0; i < 4; ++i) dst[i] = pkt[i];
         }
       }
+    }
     }
   }
 
@@ -759,12 +852,12 @@ template <int DK, int DV>
 constexpr bool kUseOneTile = DV == 64 && DK == 64;
 
 // One instance of the kernel: its shared-memory limit, the register-split check and the launch.
-template <int DK, int DV, bool SPLIT, int QT>
+template <int DK, int DV, bool SPLIT, int QT, bool DUP = false>
 int launch_instance(const AttnArgs& a, const CUtensorMap& mq, const CUtensorMap& mk,
                     const CUtensorMap& mv, const SplitPlan& sp, float* ws_o, float2* ws_ml, char* msg,
                     size_t msglen) {
-  using C = Cfg<DK, DV, QT>;
-  auto kern = attn_fwd_bf16_tc_kernel<DK, DV, SPLIT, QT>;
+  using C = Cfg<DK, DV, QT, DUP>;
+  auto kern = attn_fwd_bf16_tc_kernel<DK, DV, SPLIT, QT, DUP>;
   const cudaError_t attr_err = ensure_smem_limit(reinterpret_cast<const void*>(kern), C::kSmemBytes);
   if (attr_err != cudaSuccess) {
     snprintf(msg, msglen, "cudaFuncSetAttribute (bf16 kernel): %s", cudaGetErrorString(attr_err));
@@ -790,7 +883,7 @@ int launch_instance(const AttnArgs& a, const CUtensorMap& mq, const CUtensorMap&
       return 5;
     }
   }
-  const int64_t n_qblocks = (a.Nq + QT * kBM - 1) / (QT * kBM);
+  const int64_t n_qblocks = (a.Nq + C::kQLoads * kBM - 1) / (C::kQLoads * kBM);
   const int64_t grid = a.B * a.H * n_qblocks * sp.n_splits;
   if (grid > 0x7fffffffLL) {
     snprintf(msg, msglen, "bf16 path: %lld CTAs exceeds the grid limit", (long long)grid);
@@ -830,8 +923,27 @@ int launch_tc(const AttnArgs& a, const CUtensorMap& mq, const CUtensorMap& mk,
   const int64_t rows = a.B * a.H * a.Nq;
   float* ws_o = static_cast<float*>(ws);
   float2* ws_ml = reinterpret_cast<float2*>(ws_o + sp.n_splits * rows * DV);
-  const int rc = one ? launch_instance<DK, DV, true, 1>(a, mq, mk, mv, sp, ws_o, ws_ml, msg, msglen)
-                     : launch_instance<DK, DV, true, 2>(a, mq, mk, mv, sp, ws_o, ws_ml, msg, msglen);
+  // One tile's rows on both tiles' pipelines (DUP) where d_v = 64 leaves tensor memory for two S
+  // buffers.  At d = 64 two one-tile CTAs share an SM instead once the grid is past one per SM.  Two
+  // one-tile CTAs -> DUP on a GB300: 1x32x128x16384 (4 splits) 41.3 -> 32.5 us, 11x1x11x20680 (13
+  // splits) 20.9 -> 16.6, 1x1x1x65536 (25 splits) 28.7 -> 21.1; 2x40x3x9000 (240 CTAs) 39.7 -> 43.6.
+  int sms = 0;
+  if constexpr (DV == 64) {
+    const cudaError_t se = device_sm_count(&sms);
+    if (se != cudaSuccess) {
+      snprintf(msg, msglen, "SM count of the current device: %s", cudaGetErrorString(se));
+      return 5;
+    }
+  }
+  int rc;
+  if (!one) {
+    rc = launch_instance<DK, DV, true, 2>(a, mq, mk, mv, sp, ws_o, ws_ml, msg, msglen);
+  } else if (DV == 64 && (DK == 128 || a.B * a.H * sp.n_splits <= sms)) {
+    if constexpr (DV == 64)
+      rc = launch_instance<DK, DV, true, 2, true>(a, mq, mk, mv, sp, ws_o, ws_ml, msg, msglen);
+  } else {
+    rc = launch_instance<DK, DV, true, 1>(a, mq, mk, mv, sp, ws_o, ws_ml, msg, msglen);
+  }
   if (rc != 0) return rc;
   const long long blocks = (rows + 7) / 8;
   const cudaError_t e = launch_dependent(splitkv_merge_kernel<DV>, dim3(unsigned(blocks)), dim3(256), 0,
