@@ -48,7 +48,7 @@ struct BwdShape {
 // Two groups always: a group's sums decide the last bits of a (b, h) slice, which must not depend on
 // how many slices a call has.
 constexpr BwdShape kTiles[] = {
-    {4, 4, 2, 13.2f, 13.2f}, {4, 2, 2, 8.3f, 6.9f}, {2, 2, 2, 5.7f, 5.0f}, {1, 2, 2, 5.0f, 3.5f}};
+    {4, 4, 2, 13.2f, 13.2f}, {4, 2, 2, 8.3f, 7.4f}, {2, 2, 2, 5.7f, 5.0f}, {1, 2, 2, 5.0f, 3.5f}};
 size_t bwd_smem(const BwdShape& t, int dk, int dv) {
   const size_t rows = 4 * size_t(t.r) * t.wr, step = size_t(kBN) * t.kw;
   const size_t d = odd_stride(dk) + odd_stride(dv), cols = (dk > dv ? dk : dv) > 64 ? 128 : 64;
@@ -360,7 +360,7 @@ cudaError_t launch_rows(const BwdArgs& a, const float* Lw, const float* Dw, int6
       int(a.Nk), int(nq_pad), int(a.dk), int(a.dv), unsigned(BH * n_kt), int(n_kt), int(n_qt), a.scale);
 }
 
-// The shape with the least estimated time: all CTAs' steps spread over the SMs plus half of the
+// The shape with the least estimated time: all CTAs' steps spread over the SMs plus a third of the
 // longest CTA, and at least that CTA's own chain (within 10 % of the measured times of 18 sizes).
 int pick_tile(const BwdArgs& a, int sms) {
   const double bh = double(a.B * a.H);
@@ -376,7 +376,7 @@ int pick_tile(const BwdArgs& a, int sms) {
     const double kv = 8.0 / 7 * double((a.Nq + step - 1) / step), q = 6.0 / 7 * double((a.Nk + step - 1) / step);
     const double ctas_kv = bh * double((a.Nk + rows - 1) / rows), ctas_q = bh * double((a.Nq + rows - 1) / rows);
     const double chain = (kv > q ? kv : q) * t.lone;
-    double time = (ctas_kv * kv + ctas_q * q) * (two ? t.shared : t.lone) / sms + 0.5 * chain;
+    double time = (ctas_kv * kv + ctas_q * q) * (two ? t.shared : t.lone) / sms + 0.35 * chain;
     if (time < chain) time = chain;
     if (best < 0 || time < best_time) {
       best = i;
