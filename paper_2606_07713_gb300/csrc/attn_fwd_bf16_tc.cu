@@ -194,6 +194,7 @@ attn_fwd_bf16_tc_kernel(const __grid_constant__ CUtensorMap tmQ,
                         int Nq, int Nk, int n_qblocks, float c_log2, uint64_t wait_limit_ns,
                         int n_splits, int kv_per_split, float* __restrict__ ws_o,
                         float2* __restrict__ ws_ml, float* __restrict__ lse) {
+  static_assert(SPLIT || !DUP, "DUP writes partials");
   using C = Cfg<DK, DV, QT, DUP>;
   constexpr int kQTiles = QT;
   constexpr int kStep = DUP ? 2 : 1;             // a tile takes every kStep-th key block
@@ -452,6 +453,9 @@ attn_fwd_bf16_tc_kernel(const __grid_constant__ CUtensorMap tmQ,
     float l = 0.f;        // running sum of exp2(c_log2 * s - m)
     bool ok = true;
     const int n_mine = DUP ? (n_kt - j + 1) / 2 : n_kt;
+    // What the exponents subtract.  DUP: a tile whose keys so far all score -inf (a mask) must not
+    // turn into NaN, for its partner may have the row's other keys.
+    auto shift_of = [](float mx) { return DUP && mx == -INFINITY ? 0.f : mx; };
     for (int n = 0; n < n_mine; ++n) {
       if (!wait_bounded(s_full(j), uint32_t(n) & 1u, wc)) {
         ok = false;
@@ -487,7 +491,7 @@ attn_fwd_bf16_tc_kernel(const __grid_constant__ CUtensorMap tmQ,
         const bool need = m_tile > m + kRescaleLog2;
         if (__any_sync(0xffffffffu, need)) {
           const float m_new = fmaxf(m, m_tile);
-          alpha = ex2_approx(m - m_new);
+          alpha = ex2_approx(m - shift_of(m_new));
           l *= alpha;
           m = m_new;
           rescale = true;
@@ -496,7 +500,7 @@ attn_fwd_bf16_tc_kernel(const __grid_constant__ CUtensorMap tmQ,
       // Step II + III: p = exp2(c*s - m), row sum, P -> bf16 pairs into P_j's TMEM columns
       // (chunk c of 32 scores becomes 16 packed columns at column 16c of P_j).
       const uint64_t cc = pack_f32x2(c_log2, c_log2);
-      const uint64_t mm = pack_f32x2(-m, -m);
+      const uint64_t mm = pack_f32x2(-shift_of(m), -shift_of(m));
       float l0 = 0.f, l1 = 0.f, l2 = 0.f, l3 = 0.f;
       const bool full = valid == kBN;
       // Chunk c of 32 scores -> p = exp2(c*s - m), row sums, bf16 pairs in pk.
@@ -586,12 +590,8 @@ attn_fwd_bf16_tc_kernel(const __grid_constant__ CUtensorMap tmQ,
       const int grow = q0 + row;
       if (j == 0 && ok && wait_bounded(o_done(0), 0, wc)) {
         tc_fence_after_sync();
-        const float inv_l = SPLIT ? 1.0f : 1.0f / l;
-        if (!SPLIT && lse != nullptr && grow < Nq)
-          lse[size_t(bh) * Nq + grow] = (m + lg2_approx(l)) * 0.69314718055994531f;
-        const size_t prow =
-            SPLIT ? (size_t(*split_s) * (gridDim.x / n_splits / n_qblocks) + bh) * Nq + grow : 0;
-        if (SPLIT && grow < Nq) ws_ml[prow] = make_float2(m, l);
+        const size_t prow = (size_t(*split_s) * (gridDim.x / n_splits / n_qblocks) + bh) * Nq + grow;
+        if (grow < Nq) ws_ml[prow] = make_float2(m, l);
 #pragma unroll
         for (int c = 0; c < DV; c += 16) {
           uint32_t o[16];
@@ -605,20 +605,10 @@ attn_fwd_bf16_tc_kernel(const __grid_constant__ CUtensorMap tmQ,
             if (both) v[i] = fmaf(mrg[(2 + c + i) * kBM + row], w1, v[i]);
           }
           if (grow < Nq) {
-            if constexpr (SPLIT) {
-              float4* dst = reinterpret_cast<float4*>(ws_o + prow * DV + c);
+            float4* dst = reinterpret_cast<float4*>(ws_o + prow * DV + c);
 #pragma unroll
-              for (int i = 0; i < 4; ++i)
-                dst[i] = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
-            } else {
-              uint4* dst = reinterpret_cast<uint4*>(O + (size_t(bh) * Nq + grow) * DV + c);
-#pragma unroll
-              for (int i = 0; i < 2; ++i)
-                dst[i] = make_uint4(pack_bf16x2(v[8 * i] * inv_l, v[8 * i + 1] * inv_l),
-                                    pack_bf16x2(v[8 * i + 2] * inv_l, v[8 * i + 3] * inv_l),
-                                    pack_bf16x2(v[8 * i + 4] * inv_l, v[8 * i + 5] * inv_l),
-                                    pack_bf16x2(v[8 * i + 6] * inv_l, v[8 * i + 7] * inv_l));
-            }
+            for (int i = 0; i < 4; ++i)
+              dst[i] = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
           }
         }
       }

@@ -176,13 +176,16 @@ attn_fwd_f32_cc_kernel(const float* __restrict__ Q, const float* __restrict__ K,
         for (int j = 1; j < 8; ++j) t = fmaxf(t, s[r][j]);
 #pragma unroll
         for (int off = 8; off > 1; off >>= 1) t = fmaxf(t, __shfl_xor_sync(0xffffffffu, t, off));
-        const float mnew = fmaxf(m[r], t);         // finite: the tile has at least one key
-        const float alpha = expf(m[r] - mnew);     // exp(-inf) = 0 on the first tile
+        const float mnew = fmaxf(m[r], t);
+        // A group whose keys so far all score -inf (a mask) must not turn into NaN, for the other
+        // groups may have the row's other keys.
+        const float shift = mnew == -INFINITY ? 0.f : mnew;
+        const float alpha = expf(m[r] - shift);    // exp(-inf) = 0 on the first tile
         m[r] = mnew;
         float sum = 0.f;
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
-          s[r][j] = expf(s[r][j] - mnew);
+          s[r][j] = expf(s[r][j] - shift);
           sum += s[r][j];
         }
         l[r] = fmaf(l[r], alpha, sum);

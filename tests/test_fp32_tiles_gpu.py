@@ -58,3 +58,22 @@ def test_fp32_tile_edges(oracle, shape):
     assert torch.equal(o1[0, 0], o[b, h]) and torch.equal(lse1[0, 0], lse[b, h])
     for a, whole in zip(pkg.attn_bwd(*one, x.scale), grads):
         assert torch.equal(a[0, 0], whole[b, h])
+
+
+@pytest.mark.parametrize("masked", [(1, 3), (0, 2, 4), (1, 2, 3), (0, 1)])
+@pytest.mark.parametrize("nq", [9, 520])
+def test_tiles_of_masked_keys(oracle, nq, masked):
+    """Keys whose score is -inf (first feature: 1 in Q, -inf in K) have no part in the result, also
+    where a key group (64 keys of each step) has no other keys, or none in its first step."""
+    x = I.make_inputs(I.custom_config(1, 2, nq, 370, 64, 64, dtype="fp32", seed=nq + len(masked)))
+    keep = [i for i in range(370) if i // 64 not in masked]
+    x.q[..., 0] = 1.0
+    x.k[..., 0] = 0.0
+    q, k, v = to_device(x)
+    km = torch.full_like(k[..., 0], float("-inf"))
+    km[..., keep] = 0.0
+    k[..., 0] = km
+    o, lse = pkg.attn_fwd_lse(q, k, v, x.scale)
+    ref, lref = oracle.attn_lse(x.q, x.k[:, :, keep].copy(), x.v[:, :, keep].copy(), x.scale)
+    assert_close(o.cpu().numpy(), ref, "fp32", f"{nq} {masked}")
+    assert np.all(np.abs(lse.double().cpu().numpy() - lref) <= lse_bound(x, lref))

@@ -48,3 +48,36 @@ def test_merge_of_many_ranges(oracle, nq, dv):
         torch.cuda.synchronize()
         pkg.check(pkg.get_device_status())
         assert_close(o.float().cpu().numpy(), ref, "bf16", f"nq={nq} splits={splits}")
+
+
+@pytest.mark.parametrize("bh", [2, 40])
+@pytest.mark.parametrize("nk", [1029, 1280])
+def test_d64_split_small_and_large_grids(oracle, bh, nk):
+    """Two tiles on the same rows up to one CTA per SM, one-tile CTAs two to an SM past it (40 x 5
+    ranges), with an odd and an even number of key blocks in the last range."""
+    x = I.make_inputs(I.custom_config(1, bh, 7, nk, 64, 64, dtype="bf16", seed=bh + nk))
+    q, k, v = to_device(x)
+    o = pkg.attn_fwd_splitkv(q, k, v, 5, x.scale)
+    torch.cuda.synchronize()
+    pkg.check(pkg.get_device_status())
+    assert_close(o.float().cpu().numpy(), oracle.attn(x.q, x.k, x.v, x.scale), "bf16", f"{bh}x{nk}")
+
+
+@pytest.mark.parametrize("masked", [range(1, 8, 2), range(0, 8, 2), (1, 2, 3, 5), (0, 3, 4, 7)])
+@pytest.mark.parametrize("dk", [64, 128])
+def test_blocks_of_masked_keys(oracle, dk, masked):
+    """Keys whose score is -inf (first feature: 1 in Q, -inf in K) have no part in the result, also
+    where one of a CTA's two tiles has no other keys (every odd or even block of a range)."""
+    x = I.make_inputs(I.custom_config(1, 2, 50, 1024, dk, 64, dtype="bf16", seed=dk))
+    q, k, v = to_device(x)
+    q[..., 0] = 1.0
+    k[..., 0] = 0.0
+    keep = [i for i in range(1024) if i // 128 not in masked]
+    km = torch.full_like(k[..., 0], float("-inf"))
+    km[..., keep] = 0.0
+    k[..., 0] = km
+    o = pkg.attn_fwd_splitkv(q, k, v, 2, x.scale)
+    torch.cuda.synchronize()
+    pkg.check(pkg.get_device_status())
+    f = [t.float().cpu().numpy().astype("float64") for t in (q, k[:, :, keep], v[:, :, keep])]
+    assert_close(o.float().cpu().numpy(), oracle.attn(*f, x.scale), "bf16", f"{dk} {masked}")
