@@ -77,6 +77,9 @@ constexpr float kRescaleLog2 = 8.0f;  // lazy-rescale threshold: exponentials st
 // costs 4 % at d_v = 128 (1712 -> 1638 TFLOP/s on 2x32x8192^2), where the MMA issuers' waits are
 // on the critical path; the one-tile kernel ran at 709 instead of 740 with it.
 
+// Key blocks of all CTAs up to which a launch lets the next one start early (see the kernel).
+constexpr unsigned kTriggerBlocks = 1u << 15;
+
 template <int DK, int DV, int QT = 2, bool DUP = false>
 struct Cfg {
   static_assert(DK == 64 || DK == 128, "d_k must be 64 or 128");
@@ -265,11 +268,14 @@ attn_fwd_bf16_tc_kernel(const __grid_constant__ CUtensorMap tmQ,
   __syncthreads();
   tc_fence_after_sync();
   const uint32_t tmem = *tmem_slot;
-  // What follows on the stream may take SMs as they come free.  Where two CTAs share an SM this comes
-  // only after the key loop: CTAs of the next call that move in beside this one's, on whichever SMs
-  // have room, would run two to an SM with others idle (1x102x10x43657 d=64, call after call: 325 us,
-  // 402 with it here).
-  if constexpr (C::kMinBlocks == 1) launch_dependents();
+  // What follows on the stream may take SMs as they come free, in calls of up to some 300 us: the next
+  // call's CTAs then start on whichever SMs are free, out of the order in which neighbours share tiles
+  // in L2, and past that the loss is more than the launch saved (us a call, call after call, without
+  // -> with: 1x16x32768x32768 d=128 5205 -> 5238, 2x16x8192x8192 682 -> 685; 4x16x2048x2048 d=64 with
+  // the LSE 82 -> 80).  Where two CTAs share an SM this comes only after the key loop: CTAs that move
+  // in beside this one's would run two to an SM with others idle (1x102x10x43657 d=64 325 -> 402).
+  const bool trigger = n_kt <= 64 && gridDim.x * unsigned(n_kt) <= kTriggerBlocks;
+  if (C::kMinBlocks == 1 && trigger) launch_dependents();
   grid_dependency_wait();   // what came before has ended: its results are visible
 
   if (warp >= 4 * QT) {
@@ -555,8 +561,7 @@ attn_fwd_bf16_tc_kernel(const __grid_constant__ CUtensorMap tmQ,
       tc_fence_before_sync();
       mbar_arrive(p_ready(j));
     }
-    // (Past 64 key blocks, some 60 us, the launch saved is not worth the unevenness that is left.)
-    if (C::kMinBlocks > 1 && n_kt <= 64) launch_dependents();
+    if (C::kMinBlocks > 1 && trigger) launch_dependents();
     if constexpr (DUP) {
       // Merge of the two tiles' key blocks (the identity of the split merge): tile 1 leaves its m, l
       // and O in its ring, whose loads its products have all read; tile 0 takes them up.
