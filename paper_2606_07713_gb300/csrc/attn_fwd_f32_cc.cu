@@ -26,7 +26,7 @@
 //
 // Measured on a GB300 (2070 MHz; before: one lane per output column, 8-row warps, scalar loads):
 // 2x8x1000x1500 d=64 482 -> 171 us (36 TFLOP/s), 1x8x1024x1024 d=128 517 -> 125 us, 1x8x256x256
-// d=64 27 -> 10 us, 1x1x300x2048 d=64 115 -> 33 us, 1x1x128x128 d=64 10.4 -> 6.3 us.  The tile's
+// d=64 27 -> 10 us, 1x16x100x1500 133 -> 37 us, 1x1x300x2048 d=64 115 -> 33 us, 1x1x128x128 d=64 10.4 -> 4.8 us.  The tile's
 // former fill by cp.async with a zero-fill source size cost more than its products (16-row tile,
 // one 256-key step: 13 us with it, 6.4 us with the plain form and stores of zeros).
 #include <cuda_runtime.h>
