@@ -259,7 +259,8 @@ attn_fwd_f32_cc_kernel(const float* __restrict__ Q, const float* __restrict__ K,
 #pragma unroll
       for (int r = 0; r < R; ++r) {
         const float mo = other[32 * r], mn = fmaxf(m[r], mo);
-        const float a = expf(m[r] - mn), b = expf(mo - mn);
+        const float shift = mn == -INFINITY ? 0.f : mn;  // as in the loop: a later group may have keys
+        const float a = expf(m[r] - shift), b = expf(mo - shift);
         m[r] = mn;
         l[r] = fmaf(other[32 * (R + r)], b, l[r] * a);
 #pragma unroll

@@ -1,0 +1,60 @@
+"""Keys whose score is -inf (first feature: 1 in Q, -inf in K) have no part in the result, wherever
+they stand: the first key blocks of a row, every key of a key group or of a key range.  A row without
+any other key is 0/0: its output is NaN and its log-sum-exp -inf, as in any softmax."""
+import numpy as np
+import pytest
+
+from gpu_helpers import assert_close, lse_bound, to_device
+
+pytestmark = pytest.mark.gpu
+torch = pytest.importorskip("torch")
+
+import paper_2606_07713_gb300 as pkg  # noqa: E402
+from paper_2606_07713_gb300 import inputs as I  # noqa: E402
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _need_gpu():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    pkg.lib()
+
+
+def masked_inputs(shape, dtype, block, masked):
+    """Inputs whose key blocks `masked` (of `block` keys) score -inf; the oracle's inputs without them."""
+    x = I.make_inputs(I.custom_config(*shape, dtype=dtype, seed=sum(shape) + len(masked)))
+    keep = [i for i in range(shape[3]) if i // block not in masked]
+    x.q[..., 0] = 1.0
+    x.k[..., 0] = 0.0
+    q, k, v = to_device(x)
+    q[..., 0] = 1.0
+    km = torch.full_like(k[..., 0], float("-inf"))
+    km[..., keep] = 0.0
+    k[..., 0] = km
+    return x, q, k, v, (x.q, x.k[:, :, keep].copy(), x.v[:, :, keep].copy())
+
+
+def check_lse(x, lse, ref, lref):
+    # the bound of the finite keys: the masked ones add nothing to the sum of the scores' errors
+    xf = type("X", (), {"q": ref[0], "k": ref[1], "scale": x.scale})
+    assert np.all(np.abs(lse.double().cpu().numpy() - lref) <= lse_bound(xf, lref))
+
+
+@pytest.mark.parametrize("nk,masked", [(192, (0, 1)), (256, (0, 1, 2)), (370, (0, 1, 4, 5)),
+                                       (370, (0, 1, 2, 4, 5)), (500, (0, 1, 2, 3))])
+@pytest.mark.parametrize("nq", [9, 520])
+def test_fp32_key_groups_without_a_key(oracle, nq, nk, masked):
+    """Blocks of 64 keys, as the key groups take them: two, three and four empty groups of four."""
+    x, q, k, v, ref = masked_inputs((1, 2, nq, nk, 64, 64), "fp32", 64, masked)
+    o, lse = pkg.attn_fwd_lse(q, k, v, x.scale)
+    oref, lref = oracle.attn_lse(*ref, x.scale)
+    assert_close(o.cpu().numpy(), oref, "fp32", f"{nq} {nk} {masked}")
+    check_lse(x, lse, ref, lref)
+
+
+@pytest.mark.parametrize("dtype,nk", [("fp32", 60), ("fp32", 300)])
+@pytest.mark.parametrize("nq", [9, 600])
+def test_no_key_at_all(nq, dtype, nk):
+    x, q, k, v, _ = masked_inputs((1, 2, nq, nk, 64, 64), dtype, nk, (0,))
+    o, lse = pkg.attn_fwd_lse(q, k, v, x.scale)
+    assert torch.all(torch.isnan(o)) and torch.all(lse == float("-inf"))
