@@ -51,6 +51,7 @@
 #include <cuda_runtime.h>
 
 #include <atomic>
+#include <cfloat>
 #include <cmath>
 #include <cstdio>
 #include <mutex>
@@ -459,9 +460,6 @@ attn_fwd_bf16_tc_kernel(const __grid_constant__ CUtensorMap tmQ,
     float l = 0.f;        // running sum of exp2(c_log2 * s - m)
     bool ok = true;
     const int n_mine = DUP ? (n_kt - j + 1) / 2 : n_kt;
-    // What the exponents subtract.  DUP: a tile whose keys so far all score -inf (a mask) must not
-    // turn into NaN, for its partner may have the row's other keys.
-    auto shift_of = [](float mx) { return DUP && mx == -INFINITY ? 0.f : mx; };
     for (int n = 0; n < n_mine; ++n) {
       if (!wait_bounded(s_full(j), uint32_t(n) & 1u, wc)) {
         ok = false;
@@ -492,12 +490,15 @@ attn_fwd_bf16_tc_kernel(const __grid_constant__ CUtensorMap tmQ,
       bool rescale = false;  // warp-uniform
       float alpha = 1.f;
       if (n == 0) {
-        m = m_tile;
+        // No lower than the lowest finite value: keys that score -inf (a mask) then weigh
+        // exp2(-inf) = 0, where -inf - -inf would be NaN, and the row's other keys may come in a
+        // later block, in the other tile or in another key range.
+        m = fmaxf(m_tile, -FLT_MAX);
       } else {
         const bool need = m_tile > m + kRescaleLog2;
         if (__any_sync(0xffffffffu, need)) {
           const float m_new = fmaxf(m, m_tile);
-          alpha = ex2_approx(m - shift_of(m_new));
+          alpha = ex2_approx(m - m_new);
           l *= alpha;
           m = m_new;
           rescale = true;
@@ -506,7 +507,7 @@ attn_fwd_bf16_tc_kernel(const __grid_constant__ CUtensorMap tmQ,
       // Step II + III: p = exp2(c*s - m), row sum, P -> bf16 pairs into P_j's TMEM columns
       // (chunk c of 32 scores becomes 16 packed columns at column 16c of P_j).
       const uint64_t cc = pack_f32x2(c_log2, c_log2);
-      const uint64_t mm = pack_f32x2(-shift_of(m), -shift_of(m));
+      const uint64_t mm = pack_f32x2(-m, -m);
       float l0 = 0.f, l1 = 0.f, l2 = 0.f, l3 = 0.f;
       const bool full = valid == kBN;
       // Chunk c of 32 scores -> p = exp2(c*s - m), row sums, bf16 pairs in pk.

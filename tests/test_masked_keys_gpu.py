@@ -52,7 +52,40 @@ def test_fp32_key_groups_without_a_key(oracle, nq, nk, masked):
     check_lse(x, lse, ref, lref)
 
 
-@pytest.mark.parametrize("dtype,nk", [("fp32", 60), ("fp32", 300)])
+DIMS = [(64, 64), (128, 128), (128, 64), (64, 128)]
+
+
+@pytest.mark.parametrize("dk,dv", DIMS)
+@pytest.mark.parametrize("nq", [50, 200])
+@pytest.mark.parametrize("masked", [(0,), (0, 1, 2), (1, 2)])
+def test_first_blocks(oracle, nq, dk, dv, masked):
+    x, q, k, v, ref = masked_inputs((1, 2, nq, 500, dk, dv), "bf16", 128, masked)
+    o, lse = pkg.attn_fwd_lse(q, k, v, x.scale)
+    oref, lref = oracle.attn_lse(*ref, x.scale)
+    assert_close(o.float().cpu().numpy(), oref, "bf16", f"{nq} {dk},{dv} {masked}")
+    check_lse(x, lse, ref, lref)
+
+
+@pytest.mark.parametrize("dk,dv", DIMS)
+@pytest.mark.parametrize("nq", [50, 200])
+@pytest.mark.parametrize("masked", [range(0, 4), range(4, 8), (0, 4), (0, 1, 2, 4, 6)])
+def test_split_ranges(oracle, nq, dk, dv, masked):
+    """Two key ranges of four blocks: one of them empty, or both without their first blocks."""
+    x, q, k, v, ref = masked_inputs((1, 2, nq, 1024, dk, dv), "bf16", 128, masked)
+    o = pkg.attn_fwd_splitkv(q, k, v, 2, x.scale)
+    torch.cuda.synchronize()
+    pkg.check(pkg.get_device_status())
+    assert_close(o.float().cpu().numpy(), oracle.attn(*ref, x.scale), "bf16", f"{nq} {dk},{dv} {masked}")
+
+
+def test_split_by_the_library_past_one_cta_per_sm(oracle):
+    """80 heads in 3 ranges of d = 64: two one-tile CTAs an SM.  The first range has no key."""
+    x, q, k, v, ref = masked_inputs((2, 40, 3, 9000, 64, 64), "bf16", 128, range(0, 24))
+    o = pkg.attn_fwd_splitkv(q, k, v, pkg.MOA_SPLITS_AUTO, x.scale)
+    assert_close(o.float().cpu().numpy(), oracle.attn(*ref, x.scale), "bf16", "80 heads")
+
+
+@pytest.mark.parametrize("dtype,nk", [("fp32", 60), ("fp32", 300), ("bf16", 60), ("bf16", 300)])
 @pytest.mark.parametrize("nq", [9, 600])
 def test_no_key_at_all(nq, dtype, nk):
     x, q, k, v, _ = masked_inputs((1, 2, nq, nk, 64, 64), dtype, nk, (0,))
