@@ -139,8 +139,8 @@ __device__ __forceinline__ void bwd_rows(const float* __restrict__ A1, const flo
     request(sB2, ldv, B2, dv, k0, kStep, nB);
     if constexpr (DKDV) {
       for (int i = threadIdx.x; i < kStep; i += kThreads) {
-        const bool in = k0 + i < nB;  // padded query rows weigh exp(-inf) = 0
-        sL[i] = in ? Lw[k0 + i] : INFINITY;
+        const bool in = k0 + i < nB;
+        sL[i] = in ? Lw[k0 + i] : 0.f;
         sD[i] = in ? Dw[k0 + i] : 0.f;
       }
     }
@@ -251,10 +251,19 @@ __device__ __forceinline__ void bwd_rows(const float* __restrict__ A1, const flo
         const float Lj = DKDV ? sL[kg * kBN + col] : 0.f, Dj = DKDV ? sD[kg * kBN + col] : 0.f;
 #pragma unroll
         for (int r = 0; r < R; ++r) {
-          const float w = DKDV || col < mine ? expf(p[r][j] * scale - (DKDV ? Lj : Lr[r])) : 0.f;
+          const float w = expf(p[r][j] * scale - (DKDV ? Lj : Lr[r]));
           p[r][j] = w;
           ds[r][j] = w * (ds[r][j] - (DKDV ? Dj : Dr[r]));
         }
+      }
+      if (mine < kBN) {
+        // Streamed rows past the last are zeros, but their products need not be: 0 * inf of a key that
+        // scores -inf, or exp(0 - L) past the largest float.  They have no part in the sums.
+#pragma unroll
+        for (int r = 0; r < R; ++r)
+#pragma unroll
+          for (int j = 0; j < 8; ++j)
+            if (cg + 8 * j >= mine) p[r][j] = ds[r][j] = 0.f;
       }
       if constexpr (DKDV) accumulate(g2, p, b2, ldv);
       accumulate(g1, ds, b1, ldk);
