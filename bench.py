@@ -513,7 +513,7 @@ def run_ours_bwd(args, cfg: I.AttnConfig) -> None:
     g, gbits = I.make_grad_output(cfg)
     q, k, v, do = (to_device_bf16(b, dev) for b in (x.q_bits, x.k_bits, x.v_bits, gbits))
     o, lse = pkg.attn_fwd_lse(q, k, v, cfg.scale)
-    # d_k = d_v = 64: the one-kernel backward (5 tile products); otherwise the three-kernel one.
+    # d_k = d_v = 64: the one-kernel backward (5 tile products); otherwise the one with separate CTAs for dK/dV and dQ (7).
     # --bwd-path picks one explicitly.
     fused = args.bwd_path == "fused" or (args.bwd_path == "auto" and s.d_k == 64 and s.d_v == 64)
     wsb = pkg.moa_attn_bwd_fused_workspace_bytes if fused else pkg.moa_attn_bwd_workspace_bytes
@@ -597,7 +597,7 @@ def run_ours_bwd(args, cfg: I.AttnConfig) -> None:
                 "unit": "TFLOP/s", "frac": round(achieved / peak, 4), "traffic": None,
                 "kernel": ("moa_attn_bwd_fused: attn_bwd_pre + attn_bwd_fused + attn_bwd_dq_convert"
                            if fused else
-                           "moa_attn_bwd: attn_bwd_pre + attn_bwd_dkdv + attn_bwd_dq") + " (one call)",
+                           "moa_attn_bwd: attn_bwd_pre + attn_bwd_tiles") + " (one call)",
             },
             "e2e": {
                 "value": round(whole_job_tflops(flops, args.steps, world, e2e_ms), 2),
@@ -606,7 +606,7 @@ def run_ours_bwd(args, cfg: I.AttnConfig) -> None:
                 "d2h_bytes_per_step": int(sum(t.numel() * t.element_size() for t in host_out)),
                 "api": "attn_bwd with host copies of Q, K, V, O, dO, LSE and the gradients",
             },
-            "gpu_launches": 3 * args.steps,
+            "gpu_launches": (3 if fused else 2) * args.steps,
             "clocks": clocks,
         }
         if world == 1:

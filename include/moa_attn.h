@@ -134,8 +134,8 @@ int moa_attn_fwd_lse(const void* Q, const void* K, const void* V, void* O, float
  * Supported sizes: those of moa_attn_fwd for the dtype (bf16: d_k, d_v in {64, 128}; fp32:
  * d_k, d_v <= 128 and multiples of 4).  Alignment: every tensor 16-byte aligned (LSE 4-byte).
  * Outputs and workspace must not overlap each other or any input.
- * Behaviour: asynchronous; three kernel launches on `stream` (per-row D and LSE in log2
- * units, then dK/dV and dQ in either order; fp32: one launch for both).  Allocates nothing.  Bounded waits as for moa_attn_fwd
+ * Behaviour: asynchronous; two kernel launches on `stream` (per-row D and LSE, for bf16 in log2
+ * units; then dK, dV and dQ).  Allocates nothing.  Bounded waits as for moa_attn_fwd
  * (moa_get_device_status reports a timeout).  bf16: accumulation is fp32 in tensor memory and
  * the weights W and dS enter the tensor-core products rounded to bf16.  fp32: every step in
  * fp32 (expf for the weights).
@@ -171,7 +171,7 @@ size_t moa_attn_bwd_workspace_bytes(int64_t B, int64_t H, int64_t N_q, int64_t N
  * Errors: those of moa_attn_bwd; MOA_ERR_UNSUPPORTED_DTYPE for fp32, MOA_ERR_UNSUPPORTED_SHAPE
  * for other head dimensions.
  * Behaviour: asynchronous; three kernel launches on `stream` (per-row D and LSE with the
- * accumulator zeroed, the tile kernel, the dQ conversion), or moa_attn_bwd's three where those are
+ * accumulator zeroed, the tile kernel, the dQ conversion), or moa_attn_bwd's two where those are
  * estimated to take less (few key blocks or few heads).  Allocates nothing.
  */
 int moa_attn_bwd_fused(const void* Q, const void* K, const void* V, const void* O,

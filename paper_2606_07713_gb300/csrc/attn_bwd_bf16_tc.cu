@@ -9,22 +9,23 @@
 // weights are rebuilt tile by tile from the scores and the forward pass's per-row log-sum-exp,
 // W_ik = exp2(c * s_ik - LSE_i * log2 e), c = scale * log2 e.
 //
-// Three kernels, the second and third in either order and overlapping at their ends:
+// Two kernels:
 //   attn_bwd_pre_kernel   per query row: D_i and -LSE_i * log2 e into a padded fp32 workspace
 //                         (rows past N_q get D = 0 and -inf, so padded queries weigh nothing);
-//   attn_bwd_dkdv_kernel  one CTA per (b, h, block of 128 keys); streams every 128-row query
+//   attn_bwd_tiles_kernel CTAs of two kinds, those for dK and dV and those for dQ, in one launch.
+//     dkdv_cta            one CTA per (b, h, block of 128 keys); streams every 128-row query
 //                         block through a shared-memory ring and accumulates dV and dK in TMEM:
 //                           S^T = K Q^T, dP^T = V dO^T            (TMEM, fp32)
 //                           P^T = exp2(c S^T - L), dS^T = P^T (dP^T - D)   (registers, per key row)
 //                           dV += P^T dO,  dK += dS^T Q           (A operand from TMEM, bf16)
-//   attn_bwd_dq_kernel    one CTA per (b, h, block of 128 query rows); streams the key blocks:
+//     dq_cta              one CTA per (b, h, block of 128 query rows); streams the key blocks:
 //                           S = Q K^T, dP = dO V^T, dS = P (dP - D), dQ += dS K;
-//   attn_bwd_dq2_kernel   the same with 256 query rows per CTA, where the grid fills the GPU.
+//     dq2_cta             the same with 256 query rows per CTA, where the grid fills the GPU.
 // Splitting dQ from dK/dV keeps every accumulation inside one CTA (no atomics, deterministic
 // results) at the price of computing S and dP twice: 7 tile products per (query, key) block
 // pair instead of 5.
 //
-// CTA organisation of both tile kernels (one CTA per SM: 512 TMEM columns):
+// CTA organisation of dkdv_cta and dq_cta (one CTA per SM: 512 TMEM columns):
 //   warps 0..4P-1: 128 rows x P column parts (P = 4 for d_k + d_v = 128, else 2).  Warp w owns
 //              TMEM lanes 32*(w%4).. (its rows) and columns [(128/P)*(w/4), +128/P) of the
 //              128-wide score tiles; it writes its bf16 P or dS back into the first half of those
@@ -144,18 +145,18 @@ __device__ __forceinline__ void store_row_bf16(uint32_t taddr, float mul, __nv_b
   }
 }
 
-// The dK/dV and dQ kernels depend on the per-row kernel, not on each other, and the second of the two
-// launched takes the SMs that the first one's last round leaves idle.  The first waits for the per-row
-// kernel before it lets dependents start; so the second needs no wait of its own (it reads the per-row
-// values through L2).  Its end has to stand for the first one's too: one CTA of it, the last, ends
-// only after that grid (all of them waiting would hold SMs idle until then).
-__device__ __forceinline__ void tile_kernel_begin(bool second) {
-  if (!second) grid_dependency_wait();
-  launch_dependents();
-}
-__device__ __forceinline__ void tile_kernel_end(bool second) {
-  if (second && blockIdx.x == gridDim.x - 1) grid_dependency_wait();
-}
+// What the CTAs of the tile kernel work on.
+struct TileArgs {
+  const float* nL;  // per padded query row: -LSE * log2 e
+  const float* Dd;  // and D
+  __nv_bfloat16 *dQ, *dK, *dV;
+  int Nq, Nk, Nq_pad;
+  int n_kblocks, n_qblocks;  // CTAs per (b, h) slice: for dK and dV, for dQ
+  unsigned n_first;          // CTAs [0, n_first) are of one kind, the rest of the other
+  bool dkdv_first;
+  float c_log2, scale;
+  uint64_t wait_limit_ns;
+};
 
 // ------------------------------------------------------------------------------------------
 // Per-row preprocessing
@@ -215,8 +216,8 @@ attn_bwd_pre_kernel(const __nv_bfloat16* __restrict__ O, const __nv_bfloat16* __
 // ------------------------------------------------------------------------------------------
 // dK and dV: one CTA per (b, h, 128-key block)
 // ------------------------------------------------------------------------------------------
-template <int DK, int DV>
-struct DkDvCfg : Warps<bwd_parts(DK, DV)> {
+template <int DK, int DV, int P>
+struct DkDvCfg : Warps<P> {
   static_assert((DK == 64 || DK == 128) && (DV == 64 || DV == 128), "d_k, d_v in {64, 128}");
   static constexpr int kKBytes = kBlk * DK * 2;
   static constexpr int kVBytes = kBlk * DV * 2;
@@ -239,15 +240,16 @@ struct DkDvCfg : Warps<bwd_parts(DK, DV)> {
   static_assert(kSmemBytes <= 232448, "shared memory budget");
 };
 
-template <int DK, int DV>
-__global__ void __launch_bounds__(DkDvCfg<DK, DV>::kThreads, 1)
-attn_bwd_dkdv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
-                     const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmDO,
-                     const float* __restrict__ nL, const float* __restrict__ Dd,
-                     __nv_bfloat16* __restrict__ dK, __nv_bfloat16* __restrict__ dV, int Nk,
-                     int Nq_pad, int n_kblocks, float c_log2, float scale, bool second,
-                     uint64_t wait_limit_ns) {
-  using C = DkDvCfg<DK, DV>;
+template <int DK, int DV, int P>
+__device__ __forceinline__ void dkdv_cta(const CUtensorMap& tmQ, const CUtensorMap& tmK,
+                                         const CUtensorMap& tmV, const CUtensorMap& tmDO,
+                                         const TileArgs& a, unsigned cta) {
+  using C = DkDvCfg<DK, DV, P>;
+  const float *nL = a.nL, *Dd = a.Dd;
+  __nv_bfloat16 *dK = a.dK, *dV = a.dV;
+  const int Nk = a.Nk, Nq_pad = a.Nq_pad, n_kblocks = a.n_kblocks;
+  const float c_log2 = a.c_log2, scale = a.scale;
+  const uint64_t wait_limit_ns = a.wait_limit_ns;
   constexpr int kParts = C::kParts, kCols = C::kCols, kComputeThreads = C::kComputeThreads;
   constexpr int kMmaWarp = C::kMmaWarp, kLoadWarp = C::kLoadWarp;
   extern __shared__ uint8_t smem_raw[];
@@ -267,8 +269,8 @@ attn_bwd_dkdv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
 
   const int warp = threadIdx.x >> 5;
   const int lane = threadIdx.x & 31;
-  const int bh = blockIdx.x / n_kblocks;
-  const int k0 = (blockIdx.x % n_kblocks) * kBlk;
+  const int bh = cta / n_kblocks;
+  const int k0 = (cta % n_kblocks) * kBlk;
   const int n_qb = Nq_pad / kBlk;
   const WaitCtl wc{abort_flag, wait_limit_ns, 0u, &g_moa_bwd_status};
 
@@ -294,7 +296,8 @@ attn_bwd_dkdv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
   __syncthreads();
   tc_fence_after_sync();
   const uint32_t tmem = *tmem_slot;
-  tile_kernel_begin(second);
+  launch_dependents();     // what follows on the stream may take SMs as they come free
+  grid_dependency_wait();  // what came before has ended: its results are visible
 
   if (warp == kLoadWarp) {
     // ---------------------------------------------------------------- TMA producer
@@ -428,7 +431,7 @@ attn_bwd_dkdv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
       // it is freed even on the abort path.
       mma_commit(acc_done);
     }
-  } else {
+  } else if (warp < kMmaWarp) {
     // ---------------------------------------------------------------- compute warps
     const int part = warp >> 2;              // column part of the 128-query tiles
     const int lane_base = (warp & 3) * 32;   // TMEM lanes (key rows) of this warp
@@ -522,7 +525,6 @@ attn_bwd_dkdv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
     tc_fence_after_sync();
     tmem_dealloc(tmem, kTmemCols);
   }
-  tile_kernel_end(second);
 }
 
 // ------------------------------------------------------------------------------------------
@@ -551,13 +553,15 @@ struct DqCfg : Warps<bwd_parts(DK, DV)> {
 };
 
 template <int DK, int DV>
-__global__ void __launch_bounds__(DqCfg<DK, DV>::kThreads, 1)
-attn_bwd_dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
-                   const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmDO,
-                   const float* __restrict__ nL, const float* __restrict__ Dd,
-                   __nv_bfloat16* __restrict__ dQ, int Nq, int Nk, int Nq_pad, int n_qblocks,
-                   float c_log2, float scale, bool second, uint64_t wait_limit_ns) {
+__device__ __forceinline__ void dq_cta(const CUtensorMap& tmQ, const CUtensorMap& tmK,
+                                       const CUtensorMap& tmV, const CUtensorMap& tmDO,
+                                       const TileArgs& a, unsigned cta) {
   using C = DqCfg<DK, DV>;
+  const float *nL = a.nL, *Dd = a.Dd;
+  __nv_bfloat16* dQ = a.dQ;
+  const int Nq = a.Nq, Nk = a.Nk, Nq_pad = a.Nq_pad, n_qblocks = a.n_qblocks;
+  const float c_log2 = a.c_log2, scale = a.scale;
+  const uint64_t wait_limit_ns = a.wait_limit_ns;
   constexpr int kCols = C::kCols, kComputeThreads = C::kComputeThreads;
   constexpr int kMmaWarp = C::kMmaWarp, kLoadWarp = C::kLoadWarp;
   extern __shared__ uint8_t smem_raw[];
@@ -577,8 +581,8 @@ attn_bwd_dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
 
   const int warp = threadIdx.x >> 5;
   const int lane = threadIdx.x & 31;
-  const int bh = blockIdx.x / n_qblocks;
-  const int q0 = (blockIdx.x % n_qblocks) * kBlk;
+  const int bh = cta / n_qblocks;
+  const int q0 = (cta % n_qblocks) * kBlk;
   const int n_kb = (Nk + kBlk - 1) / kBlk;
   const WaitCtl wc{abort_flag, wait_limit_ns, 0u, &g_moa_bwd_status};
 
@@ -604,7 +608,8 @@ attn_bwd_dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
   __syncthreads();
   tc_fence_after_sync();
   const uint32_t tmem = *tmem_slot;
-  tile_kernel_begin(second);
+  launch_dependents();     // what follows on the stream may take SMs as they come free
+  grid_dependency_wait();  // what came before has ended: its results are visible
 
   if (warp == kLoadWarp) {
     // ---------------------------------------------------------------- TMA producer
@@ -727,7 +732,7 @@ attn_bwd_dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
     const uint32_t tS = tmem + lanes + C::kTmemS + part * kCols;
     const uint32_t tDP = tmem + lanes + C::kTmemDP + part * kCols;
     const size_t vrow = size_t(bh) * Nq_pad + size_t(q0 + row);  // padded: always in range
-    const float nl = __ldcg(nL + vrow), dd = __ldcg(Dd + vrow);
+    const float nl = nL[vrow], dd = Dd[vrow];
     const uint64_t cc = pack_f32x2(c_log2, c_log2);
     const uint64_t nn = pack_f32x2(nl, nl);
     bool ok = true;
@@ -780,9 +785,7 @@ attn_bwd_dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
     tc_fence_after_sync();
     tmem_dealloc(tmem, kTmemCols);
   }
-  tile_kernel_end(second);
 }
-
 
 // ------------------------------------------------------------------------------------------
 // dQ, two query tiles per CTA: one CTA per (b, h, 256-row query block)
@@ -824,13 +827,15 @@ struct Dq2Cfg {
 };
 
 template <int DK, int DV>
-__global__ void __launch_bounds__(Dq2Cfg<DK, DV>::kThreads, 1)
-attn_bwd_dq2_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
-                    const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmDO,
-                    const float* __restrict__ nL, const float* __restrict__ Dd,
-                    __nv_bfloat16* __restrict__ dQ, int Nq, int Nk, int Nq_pad, int n_qblocks,
-                    float c_log2, float scale, bool second, uint64_t wait_limit_ns) {
+__device__ __forceinline__ void dq2_cta(const CUtensorMap& tmQ, const CUtensorMap& tmK,
+                                        const CUtensorMap& tmV, const CUtensorMap& tmDO,
+                                        const TileArgs& a, unsigned cta) {
   using C = Dq2Cfg<DK, DV>;
+  const float *nL = a.nL, *Dd = a.Dd;
+  __nv_bfloat16* dQ = a.dQ;
+  const int Nq = a.Nq, Nk = a.Nk, Nq_pad = a.Nq_pad, n_qblocks = a.n_qblocks;
+  const float c_log2 = a.c_log2, scale = a.scale;
+  const uint64_t wait_limit_ns = a.wait_limit_ns;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                              ~uintptr_t(1023));
@@ -855,8 +860,8 @@ attn_bwd_dq2_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
 
   const int warp = threadIdx.x >> 5;
   const int lane = threadIdx.x & 31;
-  const int bh = blockIdx.x / n_qblocks;
-  const int q0 = (blockIdx.x % n_qblocks) * (2 * kBlk);
+  const int bh = cta / n_qblocks;
+  const int q0 = (cta % n_qblocks) * (2 * kBlk);
   const int n_kb = (Nk + kBlk - 1) / kBlk;
   const WaitCtl wc{abort_flag, wait_limit_ns, 0u, &g_moa_bwd_status};
 
@@ -888,7 +893,8 @@ attn_bwd_dq2_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
   __syncthreads();
   tc_fence_after_sync();
   const uint32_t tmem = *tmem_slot;
-  tile_kernel_begin(second);
+  launch_dependents();     // what follows on the stream may take SMs as they come free
+  grid_dependency_wait();  // what came before has ended: its results are visible
 
   if (warp >= 8) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(C::kRegsCtrl));
@@ -1025,7 +1031,7 @@ attn_bwd_dq2_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
     // padded rows (past the array's Nq_pad as well) weigh nothing
     const bool in = row < Nq_pad;
     const size_t vrow = size_t(bh) * Nq_pad + size_t(in ? row : 0);
-    const float nl = in ? __ldcg(nL + vrow) : -INFINITY, dd = in ? __ldcg(Dd + vrow) : 0.f;
+    const float nl = in ? nL[vrow] : -INFINITY, dd = in ? Dd[vrow] : 0.f;
     const uint64_t cc = pack_f32x2(c_log2, c_log2);
     const uint64_t nn = pack_f32x2(nl, nl);
     bool ok = true;
@@ -1093,9 +1099,40 @@ attn_bwd_dq2_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
     tc_fence_after_sync();
     tmem_dealloc(tmem, kTmemCols);
   }
-  tile_kernel_end(second);
 }
 
+// ------------------------------------------------------------------------------------------
+// The tile kernel: dK, dV and dQ in one launch
+// ------------------------------------------------------------------------------------------
+// The two kinds of CTAs depend on the per-row kernel and not on each other.  In one launch the second
+// kind fills the SMs that the first one's last round leaves idle, and every CTA waits for the per-row
+// kernel itself (as two launches the second could only overlap the first by leaving that wait out).
+template <int DK, int DV, bool TWO>
+struct TileCfg {
+  static constexpr int kParts = TWO ? 2 : bwd_parts(DK, DV);
+  using KV = DkDvCfg<DK, DV, kParts>;
+  using Q1 = DqCfg<DK, DV>;
+  using Q2 = Dq2Cfg<DK, DV>;
+  static constexpr int kThreads = TWO ? Q2::kThreads : KV::kThreads;
+  static_assert(KV::kThreads <= kThreads && (TWO || Q1::kThreads == kThreads), "CTA size");
+  static constexpr int kDqBytes = TWO ? Q2::kSmemBytes : Q1::kSmemBytes;
+  static constexpr int kSmemBytes = KV::kSmemBytes > kDqBytes ? KV::kSmemBytes : kDqBytes;
+};
+
+template <int DK, int DV, bool TWO>
+__global__ void __launch_bounds__(TileCfg<DK, DV, TWO>::kThreads, 1)
+attn_bwd_tiles_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
+                      const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmDO,
+                      const __grid_constant__ TileArgs a) {
+  const bool first = blockIdx.x < a.n_first;
+  const unsigned cta = first ? blockIdx.x : blockIdx.x - a.n_first;
+  if (first == a.dkdv_first)
+    dkdv_cta<DK, DV, TileCfg<DK, DV, TWO>::kParts>(tmQ, tmK, tmV, tmDO, a, cta);
+  else if constexpr (TWO)
+    dq2_cta<DK, DV>(tmQ, tmK, tmV, tmDO, a, cta);
+  else
+    dq_cta<DK, DV>(tmQ, tmK, tmV, tmDO, a, cta);
+}
 
 // ------------------------------------------------------------------------------------------
 // dK, dV and dQ in one kernel (d_k = d_v = 64): one CTA per (b, h, 128-key block)
@@ -1537,58 +1574,71 @@ attn_bwd_dq_convert_kernel(const float* __restrict__ dq_acc, __nv_bfloat16* __re
 // ------------------------------------------------------------------------------------------
 int64_t padded_rows(int64_t Nq) { return (Nq + kBlk - 1) / kBlk * kBlk; }
 
-// Estimated clocks of the two tile kernels of the three-kernel path: all CTAs' blocks spread over the
-// SMs plus a quarter of the longest CTA, and at least that CTA.  Per (query, key) block pair, from
-// launches that fill the GPU: dK/dV 3500, one-tile dQ 3250, two-tile dQ 4850 for two query blocks at
-// d_k + d_v > 128; 2750, 2650 and 4950 at d = 64; and 6000 to start and end a CTA.
+// Estimated clocks of a CTA of the tile kernel.  Per (query, key) block pair, from launches that fill the
+// GPU: dK/dV 3500, one-tile dQ 3250, two-tile dQ 4850 for two query blocks at d_k + d_v > 128; 2750, 2650
+// and 4950 at d = 64; and 6000 to start and end a CTA.
 template <int DK, int DV>
-double three_kernel_clocks(int64_t BH, int64_t n_qb, int64_t n_kb, int sms, bool two_tiles) {
+double dkdv_clocks(int64_t n_qb) {
+  return double(n_qb) * (DK + DV > 128 ? 3500 : 2750) + 6000;
+}
+template <int DK, int DV>
+double dq_clocks(int64_t n_kb, bool two_tiles) {
   constexpr bool kBig = DK + DV > 128;
-  constexpr double kKv = kBig ? 3500 : 2750, kOne = kBig ? 3250 : 2650, kTwo = kBig ? 4850 : 4950;
-  constexpr double kCta = 6000;
-  const double kv = double(n_qb) * kKv + kCta;
-  const double dq = double(n_kb) * (two_tiles ? kTwo : kOne) + kCta;
+  return double(n_kb) * (two_tiles ? (kBig ? 4850 : 4950) : kBig ? 3250 : 2650) + 6000;
+}
+// Of the whole tile kernel: all CTAs spread over the SMs plus a quarter of the longest, and at least that
+// CTA.
+template <int DK, int DV>
+double tiles_clocks(int64_t BH, int64_t n_qb, int64_t n_kb, int sms, bool two_tiles) {
+  const double kv = dkdv_clocks<DK, DV>(n_qb), dq = dq_clocks<DK, DV>(n_kb, two_tiles);
   const double ctas_q = double(two_tiles ? (n_qb + 1) / 2 : n_qb);
   const double chain = kv > dq ? kv : dq;
   const double t = double(BH) * (double(n_kb) * kv + ctas_q * dq) / sms + 0.25 * chain;
   return t > chain ? t : chain;
 }
 // Two query tiles per dQ CTA where that takes less.
-// Measured, one -> two tiles on a GB300: 2x16x4096x4096 d=128 788 -> 706 us, 8x8x1024x4096 d_k=128
-// d_v=64 372 -> 358, 1x16x1000x3000 d=128 90 -> 81, 4x16x2048x2048 d=64 331 -> 314; the other way round
-// 1x4x2048x2048 d=128 39 -> 49, 3x5x500x1500 d=64 22 -> 30 (too few CTAs to fill the SMs).
+// Measured, one -> two tiles on a GB300: 2x16x4096x4096 d=128 785 -> 708 us, 8x8x1024x4096 d_k=128
+// d_v=64 373 -> 357, 1x16x1000x3000 d=128 91 -> 81, 4x16x2048x2048 d=64 325 -> 307; the other way round
+// 1x4x2048x2048 d=128 37 -> 49, 3x5x500x1500 d=64 21 -> 30 (too few CTAs to fill the SMs).
 template <int DK, int DV>
 bool dq_two_tiles(int64_t BH, int64_t n_qb, int64_t n_kb, int sms) {
-  return three_kernel_clocks<DK, DV>(BH, n_qb, n_kb, sms, true) <
-         three_kernel_clocks<DK, DV>(BH, n_qb, n_kb, sms, false);
+  return tiles_clocks<DK, DV>(BH, n_qb, n_kb, sms, true) <
+         tiles_clocks<DK, DV>(BH, n_qb, n_kb, sms, false);
 }
-// Whether the three kernels take less than the fused one (d = 64): rounds of fused CTAs at 3700 clocks
+// Whether the tile kernel takes less than the fused one (d = 64): rounds of fused CTAs at 3700 clocks
 // per block pair and 7000 per CTA, its accumulator zeroed and converted; both with their launches.
-// Measured, fused / three kernels on a GB300 (us): 1x1x92x92 9.3 / 6.4, 6x8x661x84 22.1 / 15.4,
-// 3x5x500x1500 27.9 / 22.1, 1x1x8000x8000 122 / 95; 1x16x1024x1024 25.6 / 28.5, 4x16x2048x2048 255 / 314.
-bool fused_takes_three(int64_t BH, int64_t n_qb, int64_t n_kb, int sms) {
-  const double one = three_kernel_clocks<64, 64>(BH, n_qb, n_kb, sms, false);
-  const double two = three_kernel_clocks<64, 64>(BH, n_qb, n_kb, sms, true);
+// Measured, fused / tile kernel on a GB300 (us): 1x1x92x92 9.3 / 6.1, 6x8x661x84 22.1 / 14.4,
+// 3x5x500x1500 27.9 / 21.3, 1x1x8000x8000 122 / 95; 1x16x1024x1024 25.6 / 28.5, 4x16x2048x2048 255 / 307.
+bool fused_takes_tiles(int64_t BH, int64_t n_qb, int64_t n_kb, int sms) {
+  const double one = tiles_clocks<64, 64>(BH, n_qb, n_kb, sms, false);
+  const double two = tiles_clocks<64, 64>(BH, n_qb, n_kb, sms, true);
   const double rounds = double((BH * n_kb + sms - 1) / sms);
   const double fused = rounds * (double(n_qb) * 3700 + 7000) + 0.16 * double(BH * n_qb * kBlk) + 5000;
   return (one < two ? one : two) + 5200 < 0.97 * (fused + 8300);
 }
 
+// One instance of the tile kernel.
+template <int DK, int DV, bool TWO>
+cudaError_t launch_tiles(const CUtensorMap& mq, const CUtensorMap& mk, const CUtensorMap& mv,
+                         const CUtensorMap& mdo, const TileArgs& t, unsigned grid, cudaStream_t stream) {
+  using C = TileCfg<DK, DV, TWO>;
+  auto kern = attn_bwd_tiles_kernel<DK, DV, TWO>;
+  const cudaError_t e = ensure_smem_limit(reinterpret_cast<const void*>(kern), C::kSmemBytes);
+  if (e != cudaSuccess) return e;
+  return launch_dependent(kern, dim3(grid), dim3(C::kThreads), C::kSmemBytes, stream, mq, mk, mv, mdo, t);
+}
+
 template <int DK, int DV>
 int launch_bwd(const BwdArgs& a, const CUtensorMap& mq, const CUtensorMap& mk,
                const CUtensorMap& mv, const CUtensorMap& mdo, char* msg, size_t msglen) {
-  using A = DkDvCfg<DK, DV>;
-  using B = DqCfg<DK, DV>;
   const int64_t BH = a.B * a.H;
   const int64_t nq_pad = padded_rows(a.Nq);
   const int64_t n_kb = (a.Nk + kBlk - 1) / kBlk, n_qb = nq_pad / kBlk;
-  if (BH * n_kb > 0x7fffffffLL || BH * n_qb > 0x7fffffffLL || BH * nq_pad / 8 > 0x7fffffffLL ||
-      nq_pad > 0x7fffffffLL) {
+  if (BH * (n_kb + n_qb) > 0x7fffffffLL || BH * nq_pad / 8 > 0x7fffffffLL || nq_pad > 0x7fffffffLL) {
     snprintf(msg, msglen, "bf16 backward: grid too large");
     return 3;
   }
   using D = Dq2Cfg<DK, DV>;
-  const int64_t n_q2 = (n_qb + 1) / 2;
   int sms = 0;
   cudaError_t pe = device_sm_count(&sms);
   const bool two_tiles = pe == cudaSuccess && dq_two_tiles<DK, DV>(BH, n_qb, n_kb, sms);
@@ -1598,7 +1648,7 @@ int launch_bwd(const BwdArgs& a, const CUtensorMap& mq, const CUtensorMap& mk,
     static std::atomic<int> regs = {-1};
     if (regs.load(std::memory_order_relaxed) < 0) {
       cudaFuncAttributes fa;
-      pe = cudaFuncGetAttributes(&fa, reinterpret_cast<const void*>(attn_bwd_dq2_kernel<DK, DV>));
+      pe = cudaFuncGetAttributes(&fa, reinterpret_cast<const void*>(attn_bwd_tiles_kernel<DK, DV, true>));
       if (pe == cudaSuccess) regs.store(fa.numRegs, std::memory_order_relaxed);
     }
     const int r = regs.load(std::memory_order_relaxed);
@@ -1614,7 +1664,6 @@ int launch_bwd(const BwdArgs& a, const CUtensorMap& mq, const CUtensorMap& mk,
   }
   float* nL = static_cast<float*>(a.ws);
   float* Dd = nL + BH * nq_pad;
-  const float c_log2 = a.scale * kLog2e;
   const long long rows_pad = BH * nq_pad;
   constexpr int kPreRowsPerBlock = 8 * (32 / (DV / 8));
   cudaError_t e = launch_dependent(
@@ -1622,39 +1671,17 @@ int launch_bwd(const BwdArgs& a, const CUtensorMap& mq, const CUtensorMap& mk,
       dim3(256), 0, a.stream, static_cast<const __nv_bfloat16*>(a.O),
       static_cast<const __nv_bfloat16*>(a.dO), a.lse, nL, Dd, int(a.Nq), int(nq_pad), rows_pad,
       static_cast<float*>(nullptr));
-  auto launch_dkdv = [&](bool second) {
-    cudaError_t r = ensure_smem_limit(reinterpret_cast<const void*>(attn_bwd_dkdv_kernel<DK, DV>),
-                                      A::kSmemBytes);
-    if (r == cudaSuccess)
-      r = launch_dependent(attn_bwd_dkdv_kernel<DK, DV>, dim3(unsigned(BH * n_kb)), dim3(A::kThreads),
-                           A::kSmemBytes, a.stream, mq, mk, mv, mdo, static_cast<const float*>(nL),
-                           static_cast<const float*>(Dd), static_cast<__nv_bfloat16*>(a.dK),
-                           static_cast<__nv_bfloat16*>(a.dV), int(a.Nk), int(nq_pad), int(n_kb),
-                           c_log2, a.scale, second, wait_limit_ns());
-    return r;
-  };
-  auto launch_dq = [&](auto kern, int64_t blocks, int threads, int smem, bool second) {
-    cudaError_t r = ensure_smem_limit(reinterpret_cast<const void*>(kern), smem);
-    if (r == cudaSuccess)
-      r = launch_dependent(kern, dim3(unsigned(BH * blocks)), dim3(threads), smem, a.stream, mq, mk,
-                           mv, mdo, static_cast<const float*>(nL), static_cast<const float*>(Dd),
-                           static_cast<__nv_bfloat16*>(a.dQ), int(a.Nq), int(a.Nk), int(nq_pad),
-                           int(blocks), c_log2, a.scale, second, wait_limit_ns());
-    return r;
-  };
   if (e == cudaSuccess) {
-    if (two_tiles) {
-      // its CTAs run longest: first
-      e = launch_dq(attn_bwd_dq2_kernel<DK, DV>, n_q2, D::kThreads, D::kSmemBytes, false);
-      if (e == cudaSuccess) e = launch_dkdv(true);
-    } else if (n_qb >= n_kb) {  // the longer CTAs first
-      e = launch_dkdv(false);
-      if (e == cudaSuccess)
-        e = launch_dq(attn_bwd_dq_kernel<DK, DV>, n_qb, B::kThreads, B::kSmemBytes, true);
-    } else {
-      e = launch_dq(attn_bwd_dq_kernel<DK, DV>, n_qb, B::kThreads, B::kSmemBytes, false);
-      if (e == cudaSuccess) e = launch_dkdv(true);
-    }
+    const int64_t n_dq = two_tiles ? (n_qb + 1) / 2 : n_qb;
+    // the longer CTAs first
+    const bool dkdv_first = dkdv_clocks<DK, DV>(n_qb) >= dq_clocks<DK, DV>(n_kb, two_tiles);
+    TileArgs t{nL, Dd, static_cast<__nv_bfloat16*>(a.dQ), static_cast<__nv_bfloat16*>(a.dK),
+               static_cast<__nv_bfloat16*>(a.dV), int(a.Nq), int(a.Nk), int(nq_pad), int(n_kb),
+               int(n_dq), unsigned(BH * (dkdv_first ? n_kb : n_dq)), dkdv_first, a.scale * kLog2e,
+               a.scale, wait_limit_ns()};
+    const unsigned grid = unsigned(BH * (n_kb + n_dq));
+    e = two_tiles ? launch_tiles<DK, DV, true>(mq, mk, mv, mdo, t, grid, a.stream)
+                  : launch_tiles<DK, DV, false>(mq, mk, mv, mdo, t, grid, a.stream);
   }
   if (e != cudaSuccess) {
     snprintf(msg, msglen, "bf16 backward launch: %s", cudaGetErrorString(e));
@@ -1738,7 +1765,7 @@ int launch_attn_bwd_bf16_fused(const BwdArgs& a, char* msg, size_t msglen) {
     return 5;
   }
   const int64_t n_qb = (a.Nq + kBlk - 1) / kBlk, n_kb = (a.Nk + kBlk - 1) / kBlk;
-  if (fused_takes_three(BH, n_qb, n_kb, sms)) return launch_bwd<64, 64>(a, mq, mk, mv, mdo, msg, msglen);
+  if (fused_takes_tiles(BH, n_qb, n_kb, sms)) return launch_bwd<64, 64>(a, mq, mk, mv, mdo, msg, msglen);
   return launch_bwd_fused<64, 64>(a, mq, mk, mv, mdo, msg, msglen);
 }
 
