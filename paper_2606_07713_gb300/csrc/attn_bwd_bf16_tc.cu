@@ -145,6 +145,18 @@ __device__ __forceinline__ void store_row_bf16(uint32_t taddr, float mul, __nv_b
   }
 }
 
+// Zero weights for the columns from `valid` on: those past the last key or query.  Their scores come from
+// rows of zeros, but exp2(0 - L) overflows where the real scores are far below zero, and 0 * inf is the
+// score of a key masked by an infinity.  Only the last block of an axis has such columns.
+template <int COLS>
+__device__ __forceinline__ void drop_columns(float* p, int valid) {
+  if (valid < COLS) {
+#pragma unroll
+    for (int k = 0; k < COLS; ++k)
+      if (k >= valid) p[k] = 0.f;
+  }
+}
+
 // What the CTAs of the tile kernel work on.
 struct TileArgs {
   const float* nL;  // per padded query row: -LSE * log2 e
@@ -753,6 +765,7 @@ __device__ __forceinline__ void dq_cta(const CUtensorMap& tmQ, const CUtensorMap
         p[k] = ex2_approx(p[k]);
         p[k + 1] = ex2_approx(p[k + 1]);
       }
+      drop_columns<kCols>(p, Nk - j * kBlk - part * kCols);
       ok = wait_bounded(dp_full, par, wc);
       if (!ok) break;
       tc_fence_after_sync();
@@ -1051,6 +1064,7 @@ __device__ __forceinline__ void dq2_cta(const CUtensorMap& tmQ, const CUtensorMa
         p[k] = ex2_approx(p[k]);
         p[k + 1] = ex2_approx(p[k + 1]);
       }
+      drop_columns<kBlk>(p, Nk - n * kBlk);
       ok = wait_bounded(dp_full(j), par, wc);
       if (!ok) break;
       tc_fence_after_sync();
@@ -1479,6 +1493,11 @@ attn_bwd_fused_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
       tmem_wait_st();
       tc_fence_before_sync();
       mbar_arrive(p_ready);
+      // rows past the last key: their dS would enter dQ as inf * 0 (see drop_columns)
+      if (k0 + row >= Nk) {
+#pragma unroll
+        for (int q = 0; q < kCols; ++q) p[q] = 0.f;
+      }
       ok = wait_bounded(dp_full, par, wc);
       if (!ok) break;
       tc_fence_after_sync();

@@ -1,6 +1,5 @@
 """Backward at ragged lengths: the rows that complete the last tile of keys or queries weigh nothing,
-whatever the real rows hold.  Tolerances are those of the parity tests (bf16 2e-2, fp32 2e-5 of the
-largest gradient): the inputs below change no rounding, only which padded products would overflow."""
+whatever the real rows hold."""
 import numpy as np
 import pytest
 
@@ -37,6 +36,43 @@ def gradients(q, k, v, g, scale, dtype, fused):
     torch.cuda.synchronize()
     pkg.check(pkg.get_device_status())
     return lse, [x.float().cpu().numpy() for x in out]
+
+
+# (slices, N_q, N_k, d_k, d_v, fused): one- and two-tile dQ CTAs, the fused kernel
+GRIDS = [(2, 200, 129, 64, 64, False), (2, 200, 300, 128, 64, False), (160, 385, 129, 128, 128, False),
+         (160, 385, 300, 64, 128, False), (148, 300, 129, 64, 64, True), (2, 300, 1000, 64, 64, True)]
+
+
+@pytest.mark.parametrize("grid", GRIDS, ids=str)
+def test_strongly_negative_scores(grid):
+    """Q near +c and K near -c: every score is near -170, so the rows' log-sum-exp is below -88, where
+    the weight exp(0 - LSE) of a key that does not exist overflows.  The gradients are those of the same
+    call with its last block filled up by keys of weight exp(-320) = 0, bit for bit; the fused kernel's
+    dQ up to the order of its additions."""
+    bh, nq, nk, dk, dv, fused = grid
+    r = np.random.default_rng(sum(grid[:5]))
+    c = 4.5 if dk == 64 else 3.75
+    q = bf16(c + 0.25 * r.standard_normal((1, bh, nq, dk)))
+    k = bf16(-c + r.standard_normal((1, bh, nk, dk)))
+    v, g = (bf16(r.standard_normal((1, bh, n, dv))) for n in (nk, nq))
+    scale = dk ** -0.5
+    fill = -nk % 128
+    q, k, v, g = (device(a, "bf16") for a in (q, k, v, g))
+    o, lse = pkg.attn_fwd_lse(q, k, v, scale)
+    assert lse.max().item() < -100.0
+    kf = torch.cat([k, torch.full_like(k[:, :, :1], -3 * c).expand(-1, -1, fill, -1)], 2)
+    vf = torch.cat([v, torch.ones_like(v[:, :, :1]).expand(-1, -1, fill, -1)], 2)
+    got = pkg.attn_bwd(q, k, v, o, lse, g, scale, fused=fused)
+    want = pkg.attn_bwd(q, kf, vf, o, lse, g, scale, fused=fused)
+    torch.cuda.synchronize()
+    pkg.check(pkg.get_device_status())
+    assert all(torch.all(torch.isfinite(t)) for t in got)
+    if fused:
+        dq_err = (got[0].float() - want[0].float()).abs().max().item()
+        assert dq_err <= 1e-2 * want[0].float().abs().max().item()
+    else:
+        assert torch.equal(got[0], want[0])
+    assert torch.equal(got[1], want[1][:, :, :nk]) and torch.equal(got[2], want[2][:, :, :nk])
 
 
 @pytest.mark.parametrize("grid", [(2, 9, 100, 64, 64, "fp32", False), (1, 200, 300, 32, 96, "fp32", False)],
