@@ -297,6 +297,9 @@ qkv_proj_bf16_tc_kernel(const __grid_constant__ CUtensorMap tmX,
     }
   }
 
+  // All roles of this CTA have ended, so the last commit is due: the second CTA's MMA warp, which issues
+  // nothing, must not spend one wait's limit on the whole run.
+  __syncthreads();
   if (warp == kMmaWarp) wait_quiesce(drain, 0, wait_limit_ns, &g_moa_proj_status);
   tc_fence_before_sync();
   __syncwarp();
