@@ -264,6 +264,9 @@ int moa_attn_fwd_staged(const void* hQ, const void* hK, const void* hV, void* hO
  * model of the split's cost predicts a saving of at least 15 %; with a full wave of blocks or more
  * nothing is split and the call is moa_attn_fwd (same bits).  moa_attn_split_plan reports
  * the choice.
+ * Reproducibility: bitwise from run to run.  With a given number of splits a (b, h) slice has the
+ * same bits alone and in a call of any number of slices; the library's own choice of the split,
+ * and at d_k = d_v = 64 and N_q <= 128 of the kernel, follows from all sizes and the SM count.
  * MOA_FP32 has no split form: the call then computes the same result with moa_attn_fwd.
  * Errors: those of moa_attn_fwd; MOA_ERR_INVALID_ARG for num_splits < 0 or a missing, too
  * small or overlapping workspace; MOA_ERR_MISALIGNED for a misaligned workspace;

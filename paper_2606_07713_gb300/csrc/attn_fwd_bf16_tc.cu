@@ -923,6 +923,8 @@ int launch_tc(const AttnArgs& a, const CUtensorMap& mq, const CUtensorMap& mk,
   // buffers.  At d = 64 two one-tile CTAs share an SM instead once the grid is past one per SM.  Two
   // one-tile CTAs -> DUP on a GB300: 1x32x128x16384 (4 splits) 41.3 -> 32.5 us, 11x1x11x20680 (13
   // splits) 20.9 -> 16.6, 1x1x1x65536 (25 splits) 28.7 -> 21.1; 2x40x3x9000 (240 CTAs) 39.7 -> 43.6.
+  // Where the caller gives the number of splits the choice must not depend on how many slices the call
+  // has, for it decides their last bits: DUP, which loses less where it is the slower one.
   int sms = 0;
   if constexpr (DV == 64) {
     const cudaError_t se = device_sm_count(&sms);
@@ -934,7 +936,7 @@ int launch_tc(const AttnArgs& a, const CUtensorMap& mq, const CUtensorMap& mk,
   int rc;
   if (!one) {
     rc = launch_instance<DK, DV, true, 2>(a, mq, mk, mv, sp, ws_o, ws_ml, msg, msglen);
-  } else if (DV == 64 && (DK == 128 || a.B * a.H * sp.n_splits <= sms)) {
+  } else if (DV == 64 && (DK == 128 || sp.given || a.B * a.H * sp.n_splits <= sms)) {
     if constexpr (DV == 64)
       rc = launch_instance<DK, DV, true, 2, true>(a, mq, mk, mv, sp, ws_o, ws_ml, msg, msglen);
   } else {

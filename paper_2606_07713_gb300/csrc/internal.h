@@ -28,6 +28,7 @@ constexpr int64_t kQBlockRows = 256;
 struct SplitPlan {
   int n_splits = 1;
   int kv_per_split = 0x7fffffff;
+  bool given = false;  // the caller's number, not the library's choice
 };
 
 // At most `requested` splits, each of at least one key block.

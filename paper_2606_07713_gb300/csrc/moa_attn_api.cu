@@ -260,6 +260,7 @@ int choose_plan(int64_t B, int64_t H, int64_t Nq, int64_t Nk, int num_splits, in
   if (num_splits < 0) return fail(MOA_ERR_INVALID_ARG, "num_splits must be >= 0");
   if (num_splits > 0) {
     *sp = plan_splits(Nk, num_splits);
+    sp->given = true;
     return MOA_OK;
   }
   if (sms <= 0) {
