@@ -188,6 +188,17 @@ size_t moa_attn_bwd_fused_workspace_bytes(int64_t B, int64_t H, int64_t N_q, int
                                           int64_t d_k, int64_t d_v, int dtype);
 
 /*
+ * moa_attn_bwd_fused_plan -- which kernels moa_attn_bwd_fused would run (host only).
+ *
+ * For these sizes on a GPU of sm_count SMs (sm_count <= 0: the current device's count), writes
+ * *fused = 1 for the fused tile kernel and 0 for moa_attn_bwd's kernels.
+ * Errors: MOA_ERR_INVALID_ARG for sizes < 1, sizes that overflow or a null pointer; MOA_ERR_CUDA
+ * when sm_count <= 0 and no device answers.
+ */
+int moa_attn_bwd_fused_plan(int64_t B, int64_t H, int64_t N_q, int64_t N_k, int sm_count,
+                            int* fused);
+
+/*
  * moa_qkv_proj -- the input projections Q = X W_Q, K = X W_K, V = X W_V in one pass.
  *
  * Defines: paper Section 4.1 (the problem setup: Q, K, V are the input sequence X projected

@@ -19,7 +19,7 @@ from ._lib import (MOA_BF16, MOA_FP32, MoaError, check, lib, moa_attn_dnf_bytes,
                    moa_attn_fwd_splitkv, moa_attn_splitkv_workspace_bytes, moa_attn_fwd_lse,
                    moa_attn_bwd, moa_attn_bwd_workspace_bytes, moa_qkv_proj,
                    moa_attn_split_plan, MOA_SPLITS_AUTO, moa_attn_bwd_fused,
-                   moa_attn_bwd_fused_workspace_bytes)
+                   moa_attn_bwd_fused_workspace_bytes, moa_attn_bwd_fused_plan)
 
 __all__ = ["attn_fwd", "attn_fwd_staged", "get_device_status", "attn_flops", "dnf_bytes",
            "MOA_FP32", "MOA_BF16", "MoaError", "moa_attn_fwd", "moa_attn_fwd_staged",
@@ -28,7 +28,7 @@ __all__ = ["attn_fwd", "attn_fwd_staged", "get_device_status", "attn_flops", "dn
            "moa_attn_fwd_splitkv", "moa_attn_splitkv_workspace_bytes", "attn_fwd_lse",
            "moa_attn_fwd_lse", "attn_bwd", "moa_attn_bwd", "moa_attn_bwd_workspace_bytes",
            "qkv_proj", "moa_qkv_proj", "moa_attn_split_plan", "MOA_SPLITS_AUTO",
-           "moa_attn_bwd_fused", "moa_attn_bwd_fused_workspace_bytes"]
+           "moa_attn_bwd_fused", "moa_attn_bwd_fused_workspace_bytes", "moa_attn_bwd_fused_plan"]
 
 
 _torch = None  # the torch module, bound by the first call (the package imports without torch)

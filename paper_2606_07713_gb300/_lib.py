@@ -66,6 +66,8 @@ SIGNATURES = {
                                            ctypes.POINTER(ctypes.c_int),
                                            ctypes.POINTER(ctypes.c_int),
                                            ctypes.POINTER(ctypes.c_int64)]),
+    "moa_attn_bwd_fused_plan": (ctypes.c_int, [_I64, _I64, _I64, _I64, ctypes.c_int,
+                                               ctypes.POINTER(ctypes.c_int)]),
     "moa_last_error": (ctypes.c_char_p, []),
     "moa_get_device_status": (ctypes.c_int, [_VP]),
     "moa_selftest_wait_timeout": (ctypes.c_int, [ctypes.c_uint64, _VP]),
@@ -174,6 +176,13 @@ def moa_attn_split_plan(B, H, N_q, N_k, num_splits, sm_count) -> tuple[int, int,
     rc = lib().moa_attn_split_plan(B, H, N_q, N_k, num_splits, sm_count, ctypes.byref(s),
                                    ctypes.byref(per), ctypes.byref(whole))
     return rc, s.value, per.value, whole.value
+
+
+def moa_attn_bwd_fused_plan(B, H, N_q, N_k, sm_count) -> tuple[int, int]:
+    """(status, fused) of moa_attn_bwd_fused_plan."""
+    fused = ctypes.c_int(-1)
+    rc = lib().moa_attn_bwd_fused_plan(B, H, N_q, N_k, sm_count, ctypes.byref(fused))
+    return rc, fused.value
 
 
 # MOA_NOALLOC_SCRATCH_BYTES and MOA_SPLITS_AUTO of include/moa_attn.h

@@ -1765,6 +1765,10 @@ size_t bwd_fused_workspace_bytes(int64_t B, int64_t H, int64_t Nq, int64_t dk) {
   return size_t(B) * size_t(H) * size_t(padded_rows(Nq)) * sizeof(float) * size_t(2 + dk);
 }
 
+bool bwd_fused_runs_one_kernel(int64_t BH, int64_t Nq, int64_t Nk, int sms) {
+  return !fused_takes_tiles(BH, (Nq + kBlk - 1) / kBlk, (Nk + kBlk - 1) / kBlk, sms);
+}
+
 int launch_attn_bwd_bf16_fused(const BwdArgs& a, char* msg, size_t msglen) {
   if (a.dk != 64 || a.dv != 64) {
     snprintf(msg, msglen, "the fused backward supports d_k = d_v = 64; got d_k=%lld d_v=%lld",
@@ -1783,8 +1787,8 @@ int launch_attn_bwd_bf16_fused(const BwdArgs& a, char* msg, size_t msglen) {
     snprintf(msg, msglen, "fused backward set-up: %s", cudaGetErrorString(e));
     return 5;
   }
-  const int64_t n_qb = (a.Nq + kBlk - 1) / kBlk, n_kb = (a.Nk + kBlk - 1) / kBlk;
-  if (fused_takes_tiles(BH, n_qb, n_kb, sms)) return launch_bwd<64, 64>(a, mq, mk, mv, mdo, msg, msglen);
+  if (!bwd_fused_runs_one_kernel(BH, a.Nq, a.Nk, sms))
+    return launch_bwd<64, 64>(a, mq, mk, mv, mdo, msg, msglen);
   return launch_bwd_fused<64, 64>(a, mq, mk, mv, mdo, msg, msglen);
 }
 

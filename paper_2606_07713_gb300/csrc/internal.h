@@ -131,6 +131,8 @@ int launch_attn_bwd_bf16(const BwdArgs& a, char* msg, size_t msglen);
 // accumulator of padded rows x d_k after the two per-row vectors.
 size_t bwd_fused_workspace_bytes(int64_t B, int64_t H, int64_t Nq, int64_t dk);
 int launch_attn_bwd_bf16_fused(const BwdArgs& a, char* msg, size_t msglen);
+// Whether that runs the one kernel on `sms` SMs, or launch_attn_bwd_bf16's in the same workspace.
+bool bwd_fused_runs_one_kernel(int64_t BH, int64_t Nq, int64_t Nk, int sms);
 // fp32 backward on CUDA cores; same workspace layout (LSE instead of -LSE log2 e in the first half).
 int launch_attn_bwd_f32(const BwdArgs& a, char* msg, size_t msglen);
 // Reads and clears the status word of the backward kernels' bounded waits (after a sync).

@@ -558,6 +558,22 @@ size_t moa_attn_bwd_fused_workspace_bytes(int64_t B, int64_t H, int64_t N_q, int
   return moa::bwd_fused_workspace_bytes(B, H, N_q, d_k);
 }
 
+int moa_attn_bwd_fused_plan(int64_t B, int64_t H, int64_t N_q, int64_t N_k, int sm_count,
+                            int* fused) {
+  if (B <= 0 || H <= 0 || N_q <= 0 || N_k <= 0)
+    return moa::fail(MOA_ERR_INVALID_ARG, "sizes must be positive");
+  if (fused == nullptr) return moa::fail(MOA_ERR_INVALID_ARG, "null pointer");
+  if (moa::numel4(B, H, N_q, 64) < 0 || moa::numel4(B, H, N_k, 64) < 0)
+    return moa::fail(MOA_ERR_INVALID_ARG, "sizes overflow");
+  if (sm_count <= 0) {
+    const int rc = moa::current_sm_count(&sm_count);
+    if (rc != MOA_OK) return rc;
+  }
+  *fused = moa::bwd_fused_runs_one_kernel(B * H, N_q, N_k, sm_count) ? 1 : 0;
+  moa::t_last_error[0] = '\0';
+  return MOA_OK;
+}
+
 int moa_qkv_proj(const void* X, const void* W, void* Q, void* K, void* V, int64_t B, int64_t N,
                  int64_t d_model, int64_t H, int64_t d_k, int64_t d_v, int dtype, void* stream) {
   if (!X || !W || !Q || !K || !V) return moa::fail(MOA_ERR_INVALID_ARG, "null tensor pointer");
