@@ -86,7 +86,7 @@ attn_bwd_f32_pre_kernel(const float* __restrict__ O, const float* __restrict__ d
 }
 
 // Column blocks of 32 (C) cover both d_k and d_v.  R: rows per thread (4R per warp).  WR: row
-// warps, KW: groups of the streamed axis.
+// warps, KW: groups of the streamed axis (two or more).
 template <int C, int R, int WR, int KW>
 struct BwdTile {
   static constexpr int kThreads = 32 * WR * KW;
@@ -241,7 +241,7 @@ __device__ __forceinline__ void bwd_rows(const float* __restrict__ A1, const flo
     const int mine = int(left) - kg * kBN;  // streamed rows from this group's tile on
     cp_async_wait<0>();
     __syncthreads();
-    if (KW == 1 || mine > 0) {
+    if (mine > 0) {
       float p[R][8], ds[R][8];
       dots(p, a1, b1, ldk, dk);
       dots(ds, a2, b2, ldv, dv);
@@ -273,34 +273,32 @@ __device__ __forceinline__ void bwd_rows(const float* __restrict__ A1, const flo
   }
 
   launch_dependents();  // not before: see the bf16 forward on CTAs that share an SM
-  if constexpr (KW > 1) {
-    // Sum over the groups, in their order: groups g > 0 leave theirs where the tiles were
-    // (thread-private slots, lane-contiguous).
-    constexpr int kState = (DKDV ? 2 : 1) * 4 * R * C;
-    float* slot = sB1 + warp * kState * 32 + lane;
-    if (kg > 0) {
-      float* mine = slot + (kg - 1) * WR * kState * 32;
+  // Sum over the groups, in their order: groups g > 0 leave theirs where the tiles were
+  // (thread-private slots, lane-contiguous).
+  constexpr int kState = (DKDV ? 2 : 1) * 4 * R * C;
+  float* slot = sB1 + warp * kState * 32 + lane;
+  if (kg > 0) {
+    float* mine = slot + (kg - 1) * WR * kState * 32;
 #pragma unroll
-      for (int r = 0; r < R; ++r)
+    for (int r = 0; r < R; ++r)
 #pragma unroll
-        for (int c = 0; c < 4 * C; ++c) {
-          mine[32 * (4 * C * r + c)] = g1[r][c];
-          if (DKDV) mine[32 * (4 * R * C + 4 * C * r + c)] = g2[DKDV ? r : 0][c];
-        }
-    }
-    __syncthreads();
-    if (kg > 0) return;
+      for (int c = 0; c < 4 * C; ++c) {
+        mine[32 * (4 * C * r + c)] = g1[r][c];
+        if (DKDV) mine[32 * (4 * R * C + 4 * C * r + c)] = g2[DKDV ? r : 0][c];
+      }
+  }
+  __syncthreads();
+  if (kg > 0) return;
 #pragma unroll 1
-    for (int g = 0; g < KW - 1; ++g) {
-      const float* other = slot + g * WR * kState * 32;
+  for (int g = 0; g < KW - 1; ++g) {
+    const float* other = slot + g * WR * kState * 32;
 #pragma unroll
-      for (int r = 0; r < R; ++r)
+    for (int r = 0; r < R; ++r)
 #pragma unroll
-        for (int c = 0; c < 4 * C; ++c) {
-          g1[r][c] += other[32 * (4 * C * r + c)];
-          if (DKDV) g2[DKDV ? r : 0][c] += other[32 * (4 * R * C + 4 * C * r + c)];
-        }
-    }
+      for (int c = 0; c < 4 * C; ++c) {
+        g1[r][c] += other[32 * (4 * C * r + c)];
+        if (DKDV) g2[DKDV ? r : 0][c] += other[32 * (4 * R * C + 4 * C * r + c)];
+      }
   }
 #pragma unroll
   for (int r = 0; r < R; ++r) {

@@ -50,7 +50,7 @@ constexpr int kLdp = kHalf + 8;             // floats per row of P: 4 rows of a 
 constexpr int kMaxSmem = 232448;            // shared memory a CTA can have
 
 // VC: 32-column blocks of V (ceil(d_v / 32)).  R: rows per thread (4R per warp).  WR: row warps,
-// KW: key groups.
+// KW: key groups (two or more).
 template <int VC, int R, int WR, int KW>
 struct F32Tile {
   static constexpr int kThreads = 32 * WR * KW;
@@ -134,7 +134,7 @@ attn_fwd_f32_cc_kernel(const float* __restrict__ Q, const float* __restrict__ K,
   // left: keys from k0 on
   for (long long k0 = 0, left = Nk; left > 0; k0 += kStep, left -= kStep) {
     const int mine = int(left) - kg * kBN;  // keys from this group's tile on
-    const bool live = KW == 1 || mine > 0;  // warp-uniform
+    const bool live = mine > 0;  // warp-uniform
     cp_async_wait<1>();  // K tile (and Q) here; V may be on its way
     __syncthreads();
     float s[R][8];
@@ -235,38 +235,36 @@ attn_fwd_f32_cc_kernel(const float* __restrict__ Q, const float* __restrict__ K,
   }
 
   launch_dependents();  // not before: see the bf16 kernel on CTAs that share an SM
-  if constexpr (KW > 1) {
-    // Merge of the key groups: O = sum_g e^(m_g - M) O_g, l = sum_g e^(m_g - M) l_g, M = max m_g.
-    // Groups g > 0 leave their state where the tiles were (thread-private slots, lane-contiguous).
-    constexpr int kState = 2 * R + 4 * R * VC;
-    static_assert((KW - 1) * WR * kState * 32 <= kStep * (4 + kLdv) + kBM * KW * kLdp, "merge slots");
-    float* slot = sK + lane;
-    if (kg > 0) {
-      float* mine = slot + ((kg - 1) * WR + warp) * kState * 32;
+  // Merge of the key groups: O = sum_g e^(m_g - M) O_g, l = sum_g e^(m_g - M) l_g, M = max m_g.
+  // Groups g > 0 leave their state where the tiles were (thread-private slots, lane-contiguous).
+  constexpr int kState = 2 * R + 4 * R * VC;
+  static_assert((KW - 1) * WR * kState * 32 <= kStep * (4 + kLdv) + kBM * KW * kLdp, "merge slots");
+  float* slot = sK + lane;
+  if (kg > 0) {
+    float* mine = slot + ((kg - 1) * WR + warp) * kState * 32;
 #pragma unroll
-      for (int r = 0; r < R; ++r) {
-        mine[32 * r] = m[r];
-        mine[32 * (R + r)] = l[r];
+    for (int r = 0; r < R; ++r) {
+      mine[32 * r] = m[r];
+      mine[32 * (R + r)] = l[r];
 #pragma unroll
-        for (int c = 0; c < 4 * VC; ++c) mine[32 * (2 * R + 4 * VC * r + c)] = acc[r][c];
-      }
+      for (int c = 0; c < 4 * VC; ++c) mine[32 * (2 * R + 4 * VC * r + c)] = acc[r][c];
     }
-    __syncthreads();
-    if (kg > 0) return;
+  }
+  __syncthreads();
+  if (kg > 0) return;
 #pragma unroll 1
-    for (int g = 1; g < KW && g * kBN < Nk; ++g) {  // groups that had a key
-      const float* other = slot + ((g - 1) * WR + warp) * kState * 32;
+  for (int g = 1; g < KW && g * kBN < Nk; ++g) {  // groups that had a key
+    const float* other = slot + ((g - 1) * WR + warp) * kState * 32;
 #pragma unroll
-      for (int r = 0; r < R; ++r) {
-        const float mo = other[32 * r], mn = fmaxf(m[r], mo);
-        const float shift = mn == -INFINITY ? 0.f : mn;  // as in the loop: a later group may have keys
-        const float a = expf(m[r] - shift), b = expf(mo - shift);
-        m[r] = mn;
-        l[r] = fmaf(other[32 * (R + r)], b, l[r] * a);
+    for (int r = 0; r < R; ++r) {
+      const float mo = other[32 * r], mn = fmaxf(m[r], mo);
+      const float shift = mn == -INFINITY ? 0.f : mn;  // as in the loop: a later group may have keys
+      const float a = expf(m[r] - shift), b = expf(mo - shift);
+      m[r] = mn;
+      l[r] = fmaf(other[32 * (R + r)], b, l[r] * a);
 #pragma unroll
-        for (int c = 0; c < 4 * VC; ++c)
-          acc[r][c] = fmaf(other[32 * (2 * R + 4 * VC * r + c)], b, acc[r][c] * a);
-      }
+      for (int c = 0; c < 4 * VC; ++c)
+        acc[r][c] = fmaf(other[32 * (2 * R + 4 * VC * r + c)], b, acc[r][c] * a);
     }
   }
 #pragma unroll
