@@ -78,9 +78,6 @@ constexpr float kRescaleLog2 = 8.0f;  // lazy-rescale threshold: exponentials st
 // costs 4 % at d_v = 128 (1712 -> 1638 TFLOP/s on 2x32x8192^2), where the MMA issuers' waits are
 // on the critical path; the one-tile kernel ran at 709 instead of 740 with it.
 
-// Key blocks of all CTAs up to which a launch lets the next one start early (see the kernel).
-constexpr unsigned kTriggerBlocks = 1u << 15;
-
 template <int DK, int DV, int QT = 2, bool DUP = false>
 struct Cfg {
   static_assert(DK == 64 || DK == 128, "d_k must be 64 or 128");
@@ -269,14 +266,6 @@ attn_fwd_bf16_tc_kernel(const __grid_constant__ CUtensorMap tmQ,
   __syncthreads();
   tc_fence_after_sync();
   const uint32_t tmem = *tmem_slot;
-  // What follows on the stream may take SMs as they come free, in calls of up to some 300 us: the next
-  // call's CTAs then start on whichever SMs are free, out of the order in which neighbours share tiles
-  // in L2, and past that the loss is more than the launch saved (us a call, call after call, without
-  // -> with: 1x16x32768x32768 d=128 5205 -> 5238, 2x16x8192x8192 682 -> 685; 4x16x2048x2048 d=64 with
-  // the LSE 82 -> 80).  Where two CTAs share an SM this comes only after the key loop: CTAs that move
-  // in beside this one's would run two to an SM with others idle (1x102x10x43657 d=64 325 -> 402).
-  const bool trigger = n_kt <= 64 && gridDim.x * unsigned(n_kt) <= kTriggerBlocks;
-  if (C::kMinBlocks == 1 && trigger) launch_dependents();
   grid_dependency_wait();   // what came before has ended: its results are visible
 
   if (warp >= 4 * QT) {
@@ -562,7 +551,15 @@ attn_fwd_bf16_tc_kernel(const __grid_constant__ CUtensorMap tmQ,
       tc_fence_before_sync();
       mbar_arrive(p_ready(j));
     }
-    if (C::kMinBlocks > 1 && trigger) launch_dependents();
+    // What follows on the stream may take SMs as they come free, from here on: CTAs that move in during
+    // the key loop slow it down, and at two CTAs an SM they would run two to an SM with others idle
+    // (1x102x10x43657 d=64 325 -> 402 us).  A split kernel leaves it to its end: the merge's CTAs, and
+    // through them the next call's, gain nothing by waiting beside it.  Us a call, call after call, with
+    // the launch at the start of the loop / here / at the end: 2x16x2048x2048 d=128 53.3 / 53.4 / 53.9,
+    // 1x4x1000x1000 d=64,128 15.1 / 14.7 / 15.1, 1x16x600x20000 d=128 212.9 / 212.2 / 214.8; split
+    // 1x16x256x32768 d=128 59.8 / 59.3 / 57.5, 1x32x128x16384 d=64 32.5 / 31.5 / 29.8, 8x16x1x500 d=128
+    // 8.9 / 8.8 / 8.7.
+    if (!SPLIT) launch_dependents();
     if constexpr (DUP) {
       // Merge of the two tiles' key blocks (the identity of the split merge): tile 1 leaves its m, l
       // and O in its ring, whose loads its products have all read; tile 0 takes them up.
