@@ -152,9 +152,9 @@ struct Cfg {
   static_assert(kSmemBytes <= (kMinBlocks == 1 ? 232448 : 233472 / 2 - 1024), "shared memory budget");
 };
 
-// Maximum of 128 values (of their negations if NEG) with four independent 3-input chains.
+// Maximum of 128 values (of their negations if NEG) and `lowest` with four independent 3-input chains.
 template <bool NEG>
-__device__ __forceinline__ float row_max128(const float* s) {
+__device__ __forceinline__ float row_max128(const float* s, float lowest) {
   auto v = [&](int i) { return NEG ? -s[i] : s[i]; };
   float a0 = v(0), a1 = v(1), a2 = v(2), a3 = v(3);
 #pragma unroll
@@ -166,7 +166,7 @@ __device__ __forceinline__ float row_max128(const float* s) {
   }
   a0 = max3f(a0, v(124), v(125));
   a1 = max3f(a1, v(126), v(127));
-  return max3f(a0, a1, fmaxf(a2, a3));
+  return max3f(a0, a1, max3f(a2, a3, lowest));
 }
 
 // Multiplies DV fp32 TMEM columns of this thread's lane by alpha (warp-collective).
@@ -445,6 +445,12 @@ attn_fwd_bf16_tc_kernel(const __grid_constant__ CUtensorMap tmQ,
     const uint32_t tO = tmem + (uint32_t(lane_base) << 16) + (j ? C::kTmemO1 : C::kTmemO0);
     const uint32_t tP = tmem + (uint32_t(lane_base) << 16) + (j ? C::kTmemP1 : C::kTmemP0);
     const bool neg = c_log2 < 0.f;
+    // No maximum is below the lowest score whose scaled value is finite: keys that score -inf (a mask)
+    // then weigh exp2(-inf) = 0, where -inf - -inf would be NaN, and the row's other keys may come in a
+    // later block, in the other tile or in another key range.  A spare operand of the row maximum:
+    // raising m itself adds to every block's chain (2x16x8192x8192 d=64 with the LSE 535 -> 538 us).
+    const float c_abs = fabsf(c_log2);
+    const float lowest = c_abs > 1.f ? -FLT_MAX / c_abs * (1.f - 0x1p-22f) : -FLT_MAX;
     float m = -INFINITY;  // running maximum of c_log2 * s (log2 units)
     float l = 0.f;        // running sum of exp2(c_log2 * s - m)
     bool ok = true;
@@ -467,9 +473,9 @@ attn_fwd_bf16_tc_kernel(const __grid_constant__ CUtensorMap tmQ,
       // Step I: maximum of the scaled scores of this tile (max of s if c >= 0, else of -s).
       float tmax;
       if (valid == kBN) {
-        tmax = neg ? -row_max128<true>(s) : row_max128<false>(s);
+        tmax = neg ? -row_max128<true>(s, lowest) : row_max128<false>(s, lowest);
       } else {
-        float mx = -INFINITY;
+        float mx = lowest;
 #pragma unroll
         for (int i = 0; i < kBN; ++i)
           if (i < valid) mx = fmaxf(mx, neg ? -s[i] : s[i]);
@@ -479,10 +485,7 @@ attn_fwd_bf16_tc_kernel(const __grid_constant__ CUtensorMap tmQ,
       bool rescale = false;  // warp-uniform
       float alpha = 1.f;
       if (n == 0) {
-        // No lower than the lowest finite value: keys that score -inf (a mask) then weigh
-        // exp2(-inf) = 0, where -inf - -inf would be NaN, and the row's other keys may come in a
-        // later block, in the other tile or in another key range.
-        m = fmaxf(m_tile, -FLT_MAX);
+        m = m_tile;
       } else {
         const bool need = m_tile > m + kRescaleLog2;
         if (__any_sync(0xffffffffu, need)) {
