@@ -20,23 +20,23 @@ def _need_gpu():
     pkg.lib()
 
 
-def masked_inputs(shape, dtype, block, masked):
-    """Inputs whose key blocks `masked` (of `block` keys) score -inf; the oracle's inputs without them."""
+def masked_inputs(shape, dtype, block, masked, value=float("-inf")):
+    """Inputs whose key blocks `masked` (of `block` keys) score `value`; the oracle's inputs without them."""
     x = I.make_inputs(I.custom_config(*shape, dtype=dtype, seed=sum(shape) + len(masked)))
     keep = [i for i in range(shape[3]) if i // block not in masked]
     x.q[..., 0] = 1.0
     x.k[..., 0] = 0.0
     q, k, v = to_device(x)
     q[..., 0] = 1.0
-    km = torch.full_like(k[..., 0], float("-inf"))
+    km = torch.full_like(k[..., 0], value)
     km[..., keep] = 0.0
     k[..., 0] = km
     return x, q, k, v, (x.q, x.k[:, :, keep].copy(), x.v[:, :, keep].copy())
 
 
-def check_lse(x, lse, ref, lref):
+def check_lse(scale, lse, ref, lref):
     # the bound of the finite keys: the masked ones add nothing to the sum of the scores' errors
-    xf = type("X", (), {"q": ref[0], "k": ref[1], "scale": x.scale})
+    xf = type("X", (), {"q": ref[0], "k": ref[1], "scale": scale})
     assert np.all(np.abs(lse.double().cpu().numpy() - lref) <= lse_bound(xf, lref))
 
 
@@ -49,7 +49,7 @@ def test_fp32_key_groups_without_a_key(oracle, nq, nk, masked):
     o, lse = pkg.attn_fwd_lse(q, k, v, x.scale)
     oref, lref = oracle.attn_lse(*ref, x.scale)
     assert_close(o.cpu().numpy(), oref, "fp32", f"{nq} {nk} {masked}")
-    check_lse(x, lse, ref, lref)
+    check_lse(x.scale, lse, ref, lref)
 
 
 DIMS = [(64, 64), (128, 128), (128, 64), (64, 128)]
@@ -63,7 +63,7 @@ def test_first_blocks(oracle, nq, dk, dv, masked):
     o, lse = pkg.attn_fwd_lse(q, k, v, x.scale)
     oref, lref = oracle.attn_lse(*ref, x.scale)
     assert_close(o.float().cpu().numpy(), oref, "bf16", f"{nq} {dk},{dv} {masked}")
-    check_lse(x, lse, ref, lref)
+    check_lse(x.scale, lse, ref, lref)
 
 
 @pytest.mark.parametrize("dk,dv", DIMS)
@@ -83,6 +83,18 @@ def test_split_by_the_library_past_one_cta_per_sm(oracle):
     x, q, k, v, ref = masked_inputs((2, 40, 3, 9000, 64, 64), "bf16", 128, range(0, 24))
     o = pkg.attn_fwd_splitkv(q, k, v, pkg.MOA_SPLITS_AUTO, x.scale)
     assert_close(o.float().cpu().numpy(), oracle.attn(*ref, x.scale), "bf16", "80 heads")
+
+
+@pytest.mark.parametrize("scale", [1.5, -0.2, -1.5])
+@pytest.mark.parametrize("dtype,dk,dv", [("bf16", 64, 64), ("bf16", 128, 128), ("fp32", 64, 64)])
+def test_other_scales(oracle, dtype, dk, dv, scale):
+    """Scales of either sign, above and below 1: the masks are -inf times their sign."""
+    value = -float("inf") if scale > 0 else float("inf")
+    x, q, k, v, ref = masked_inputs((1, 2, 300, 500, dk, dv), dtype, 128, (0, 2), value)
+    o, lse = pkg.attn_fwd_lse(q, k, v, scale)
+    oref, lref = oracle.attn_lse(*ref, scale)
+    assert_close(o.float().cpu().numpy(), oref, dtype, f"{scale}")
+    check_lse(scale, lse, ref, lref)
 
 
 @pytest.mark.parametrize("dtype,nk", [("fp32", 60), ("fp32", 300), ("bf16", 60), ("bf16", 300)])
