@@ -53,7 +53,8 @@ enum moa_status {
  *     s_k        = scale * sum_{j < d_k} Q[b,h,i,j] * K[b,h,k,j]      (k < N_k)
  *     O[b,h,i,c] = sum_k exp(s_k - max_k' s_k') / (sum_k'' exp(s_k'' - max_k' s_k')) * V[b,h,k,c]
  * The softmax runs over the key axis N_k; N_q and N_k may differ, as may d_k
- * and d_v.  No mask, dropout or bias.
+ * and d_v.  No mask, dropout or bias.  A key whose score is -inf has weight 0 wherever it stands;
+ * a row of such keys only is 0/0: its O is NaN and its log-sum-exp -inf.
  *
  * Arguments:
  *   Q  device pointer, [B, H, N_q, d_k], contiguous row-major, element type dtype (read only)
@@ -138,7 +139,8 @@ int moa_attn_fwd_lse(const void* Q, const void* K, const void* V, void* O, float
  * units; then dK, dV and dQ).  Allocates nothing.  Bounded waits as for moa_attn_fwd
  * (moa_get_device_status reports a timeout).  bf16: accumulation is fp32 in tensor memory and
  * the weights W and dS enter the tensor-core products rounded to bf16.  fp32: every step in
- * fp32 (expf for the weights).
+ * fp32 (expf for the weights).  A key that scores -inf has zero dK and dV (bf16: NaN where N_q is not
+ * a multiple of 128).
  */
 int moa_attn_bwd(const void* Q, const void* K, const void* V, const void* O, const void* dO,
                  const float* LSE, void* dQ, void* dK, void* dV, int64_t B, int64_t H,

@@ -17,8 +17,8 @@
 // blocks of S and dP and R x 4C blocks of the gradients in registers; tiles, lane map and the
 // split over key groups are those of the fp32 forward kernel.
 // Measured on a GB300 (2070 MHz; before: one scalar shared load per operand and FMA, 32-row tiles):
-// 1x8x1024x1024 d=64 1014 -> 218 us (24.6 TFLOP/s of the five algorithmic products), d=128 1646 ->
-// 401 us; two iterations of the product loops together are worth 4 % of it.
+// 1x8x1024x1024 d=64 1014 -> 212 us (25.3 TFLOP/s of the five algorithmic products), d=128 1646 ->
+// 394 us; two iterations of the product loops together are worth 4 % of it.
 #include <cuda_runtime.h>
 #include <math.h>
 #include <cstdio>

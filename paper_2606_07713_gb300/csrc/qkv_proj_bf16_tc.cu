@@ -22,8 +22,8 @@
 // (status word g_moa_proj_status).  Up to 128 tokens a second kernel takes over (below).
 //
 // Measured on a GB300 against one-CTA 128 x 256 tiles with row-per-lane stores: 2x8192x4096 -> 12288
-// 1316 -> 1046 us back to back under the power cap (1253 -> 1577 TFLOP/s; 1158 -> 926 us in a burst),
-// 4x2048x1024 -> 3072 46.7 -> 43.1 us, 1x512x4096 -> 12288 57.4 -> 51.3 us.
+// 1316 -> 985 us back to back under the power cap (1253 -> 1674 TFLOP/s; 1158 -> 909 us in a burst),
+// 4x2048x1024 -> 3072 46.7 -> 42.6 us, 1x512x4096 -> 12288 57.4 -> 43.3 us.
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
@@ -320,7 +320,7 @@ qkv_proj_bf16_tc_kernel(const __grid_constant__ CUtensorMap tmX,
 // (about 100 KB of ring each) keep enough of W in flight.  Warps: 0 TMA, 1 TMEM allocation and MMA
 // issue, 2-5 epilogue (lane = column).
 // Measured on a GB300, d_model 4096 -> 12288 columns (100 MB of W), against the 256-token tile: 1
-// token 33.0 -> 16.5 us (6.1 TB/s), 40 tokens 29 -> 20 us, 128 tokens 28.7 -> 27.1 us; at 129 tokens
+// token 33.0 -> 15.9 us (6.3 TB/s), 40 tokens 29 -> 21 us, 128 tokens 28.7 -> 26.3 us; at 129 tokens
 // the tile here would need a second pass over W, so the line is at 128.
 constexpr int kSmallCols = 128;
 constexpr int kSmallThreads = 192;
